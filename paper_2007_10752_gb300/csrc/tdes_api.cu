@@ -174,6 +174,9 @@ int make_schedule(tdes::Keys24& keys, int stages, tdes_ks_t** out) {
     if (e == cudaSuccess) {
         e = tdes::launch_keysched(keys, stages, ks->tab[0], ks->tab[1], ks->chunk[0],
                                   ks->chunk[1], s);
+        if (e == cudaSuccess)  // both directions' groups are adjacent
+            e = cudaMemcpyAsync(ks->host_chunk, ks->chunk[0], sizeof ks->host_chunk,
+                                cudaMemcpyDeviceToHost, s);
         cudaError_t e2 = cudaStreamSynchronize(s);
         if (e == cudaSuccess) e = e2;
         cudaStreamDestroy(s);
@@ -229,6 +232,7 @@ void tdes_key_free(tdes_ks_t* ks) {
     if (cur != ks->device) cudaSetDevice(ks->device);
     cudaFree(ks->mem);
     if (cur >= 0 && cur != ks->device) cudaSetDevice(cur);
+    memset(ks->host_chunk, 0, sizeof ks->host_chunk);
     delete ks;
 }
 
@@ -240,7 +244,7 @@ static int ecb(const tdes_ks_t* ks, int dir, const void* in, void* out, size_t n
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     cudaError_t e;
     if (nblocks <= g_small_cutoff.load(std::memory_order_relaxed)) {
-        e = tdes::launch_small(ks->chunk[dir], ks->stages, tdes::kSmallEcb, 0, in, out, nblocks,
+        e = tdes::launch_small(tdes::small_keys(ks, dir), ks->stages, tdes::kSmallEcb, 0, in, out, nblocks,
                                kSmallThreads, s);
     } else {
         const uint64_t ntiles = (nblocks + tdes::kTileBlocks - 1) / tdes::kTileBlocks;
@@ -271,7 +275,7 @@ int tdes_ctr_crypt(const tdes_ks_t* ks, uint32_t nonce, uint32_t ctr0, const voi
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     cudaError_t e;
     if (nblocks <= g_small_cutoff.load(std::memory_order_relaxed)) {
-        e = tdes::launch_small(ks->chunk[0], ks->stages, tdes::kSmallCtr,
+        e = tdes::launch_small(tdes::small_keys(ks, 0), ks->stages, tdes::kSmallCtr,
                                (uint64_t)nonce << 32 | ctr0, in, out, nblocks, kSmallThreads, s);
     } else {
         const uint64_t ntiles = (nblocks + tdes::kTileBlocks - 1) / tdes::kTileBlocks;
@@ -291,7 +295,7 @@ int tdes_cbc_decrypt(const tdes_ks_t* ks, uint64_t iv, const void* in, void* out
     // one block per thread; in place only as a single CTA (all reads before writes)
     if (nblocks <= g_small_cutoff.load(std::memory_order_relaxed) && (in != out || nblocks <= 1024)) {
         const int threads = in != out ? kSmallThreads : (int)((nblocks + 31) / 32 * 32);
-        cudaError_t e = tdes::launch_small(ks->chunk[1], ks->stages, tdes::kSmallCbcDec, iv, in,
+        cudaError_t e = tdes::launch_small(tdes::small_keys(ks, 1), ks->stages, tdes::kSmallCbcDec, iv, in,
                                            out, nblocks, threads, s);
         return e == cudaSuccess ? TDES_OK : cuda_fail(e, "CBC-decrypt kernel launch");
     }

@@ -12,6 +12,7 @@ struct tdes_ks {
     void* mem;              // one cudaMalloc holding everything below
     uint32_t* tab[2];       // bitsliced round-constant tables: [0] encrypt, [1] decrypt
     uint8_t* chunk[2];      // scalar-path round-key groups: [0] encrypt, [1] decrypt
+    uint8_t host_chunk[2][384];  // host copies of the groups (passed to kernels by value)
 };
 
 namespace tdes {
@@ -62,10 +63,17 @@ cudaError_t launch_cbc_enc(const uint8_t* chunk_enc, int stages, uint64_t iv, co
                            void* out, uint64_t nblocks, cudaStream_t s);
 
 // One block per thread (tdes_small.cu), for calls too small to fill the GPU
-// with bitsliced tiles.  chunks: the call's scalar round-key groups of the
-// wanted direction; iv: the CBC IV, or nonce << 32 | ctr0 for CTR.
+// with bitsliced tiles.  keys: the call's scalar round-key groups of the
+// wanted direction, on the device and on the host; iv: the CBC IV, or nonce << 32 | ctr0 for CTR.
 enum SmallMode { kSmallEcb = 0, kSmallCtr = 1, kSmallCbcDec = 2 };
-cudaError_t launch_small(const uint8_t* chunks, int stages, int mode, uint64_t iv, const void* in,
+struct SmallKeys {
+    const uint8_t* dev;
+    const uint8_t* host;
+};
+inline SmallKeys small_keys(const tdes_ks* ks, int dir) {
+    return {ks->chunk[dir], ks->host_chunk[dir]};
+}
+cudaError_t launch_small(SmallKeys keys, int stages, int mode, uint64_t iv, const void* in,
                          void* out, uint64_t nblocks, int threads, cudaStream_t s);
 
 // Occupancy (CTAs per SM) of a bitsliced kernel at kWideWarps warps per CTA.

@@ -1,5 +1,7 @@
 // tdes_small.cu -- single-key calls too small to fill the GPU with bitsliced
-// tiles: one 64-bit block per thread.
+// tiles: one 64-bit block per thread, in two kernels: tdes_small_kernel (one
+// copy of the tables per CTA) and, from 28673 blocks, tdes_lanes_kernel (one
+// copy per lane, no bank conflicts).
 //
 // A bitsliced tile is 1024 blocks and costs each lane about 12 k logic
 // operations (48 rounds over 64 bit-planes), so a call of a few tiles takes
@@ -11,8 +13,12 @@
 // per CTA.
 #include <cuda_runtime.h>
 
+#include <atomic>
+#include <cstring>
+
 #include "tdes_internal.h"
 #include "tdes_keysched.cuh"
+#include "tdes_lanes.cuh"
 #include "tdes_scalar.cuh"
 
 namespace tdes {
@@ -69,16 +75,86 @@ tdes_small_kernel(const uint8_t* __restrict__ chunks, int mode, uint64_t iv, con
     }
 }
 
-cudaError_t launch_small(const uint8_t* chunks, int stages, int mode, uint64_t iv, const void* in,
+// ---- one block per thread, a copy of the tables per lane (tdes_lanes.cuh) ----
+constexpr uint64_t kLanesMinBlocks = 28672;
+
+template <int ROUNDS>
+__global__ void __launch_bounds__(512, 3)
+tdes_lanes_kernel(const __grid_constant__ LaneKeys keys, int mode, uint64_t iv, const uint8_t* in,
+                  uint8_t* out, uint32_t nblocks) {
+    extern __shared__ __align__(16) uint8_t lane_tab[];
+    const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t lane4 = (threadIdx.x & 31u) * 4u;
+    uint64_t x = 0, prev = 0;
+    if (b < nblocks) {
+        if (mode == kSmallCtr) {
+            x = (iv & 0xFFFFFFFF00000000ull) | (uint32_t)((uint32_t)iv + b);
+            prev = small_load_be(in, b);
+        } else {
+            x = small_load_be(in, b);
+            if (mode == kSmallCbcDec) prev = b ? small_load_be(in, b - 1) : iv;
+        }
+    }
+    lane_tables(lane_tab, &kSmallSP[0][0]);
+    __syncthreads();
+    if (b >= nblocks) return;
+    uint64_t y = lane_block<ROUNDS>(x, keys.w, lane4, lane_tab);
+    if (mode != kSmallEcb) y ^= prev;
+    reinterpret_cast<uint64_t*>(out)[b] = bswap64(y);
+}
+
+// Whether a call takes tdes_lanes_kernel.  Below kLanesMinBlocks the few warps
+// an SM has do not fill its shared memory's cycles and writing 64 KB of tables
+// costs more than the conflicts (16384 blocks: 6.8 us against 4.8 us of
+// tdes_small_kernel; 24576: 6.2 against 6.1; 32768: 5.1 against 6.2).  CBC
+// decryption only out of place: its CTAs write while others still read.
+static bool use_lanes(int mode, const void* in, const void* out, uint64_t nblocks) {
+    return nblocks > kLanesMinBlocks && nblocks <= (1ull << 30) &&
+           (mode != kSmallCbcDec || in != out);
+}
+
+template <int ROUNDS>
+static cudaError_t lanes_launch(const uint8_t* host_chunks, int mode, uint64_t iv, const void* in,
+                                void* out, uint32_t nblocks, cudaStream_t s) {
+    static std::atomic<uint64_t> ready{0};  // devices whose shared-memory limit is raised
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64 || !(ready.load() >> dev & 1u)) {
+        e = cudaFuncSetAttribute(tdes_lanes_kernel<ROUNDS>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kLaneTableBytes);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) ready.fetch_or(1ull << dev);
+    }
+    // CTAs of one size, as few per SM (1 to 3) as hold the call in 512 threads
+    // each: every SM gets the same share, and fewer copies of the tables to write.
+    const uint32_t per_sm = nblocks <= (uint32_t)sms * 512u ? 1u : nblocks <= (uint32_t)sms * 1024u ? 2u : 3u;
+    const uint32_t ctas = (uint32_t)sms * per_sm;
+    uint32_t threads = ((nblocks + ctas - 1) / ctas + 31u) / 32u * 32u;
+    threads = threads > 512u ? 512u : threads;
+    LaneKeys k;
+    memcpy(k.w, host_chunks, sizeof k.w);
+    tdes_lanes_kernel<ROUNDS>
+        <<<(nblocks + threads - 1) / threads, threads, kLaneTableBytes, s>>>(
+            k, mode, iv, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out), nblocks);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_small(SmallKeys keys, int stages, int mode, uint64_t iv, const void* in,
                          void* out, uint64_t nblocks, int threads, cudaStream_t s) {
+    if (use_lanes(mode, in, out, nblocks))
+        return stages == 1
+                   ? lanes_launch<16>(keys.host, mode, iv, in, out, (uint32_t)nblocks, s)
+                   : lanes_launch<48>(keys.host, mode, iv, in, out, (uint32_t)nblocks, s);
     const uint64_t grid = (nblocks + threads - 1) / threads;
     if (stages == 1)
         tdes_small_kernel<16><<<(unsigned)grid, threads, 0, s>>>(
-            chunks, mode, iv, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out),
+            keys.dev, mode, iv, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out),
             nblocks);
     else
         tdes_small_kernel<48><<<(unsigned)grid, threads, 0, s>>>(
-            chunks, mode, iv, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out),
+            keys.dev, mode, iv, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out),
             nblocks);
     return cudaGetLastError();
 }
