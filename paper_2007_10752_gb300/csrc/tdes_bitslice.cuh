@@ -181,18 +181,81 @@ TDES_HD void tdes_rounds_rt(uint32_t (&Lh)[32], uint32_t (&Rh)[32], const uint32
     TDES_KEY_PASS(TDES_EPI, TDES_TABLE_EPI);
 }
 
+// All bits of the word equal to bit 8 * byte + 7 of x (a byte permute in its
+// sign-replicating mode).
+template <int BYTE>
+TDES_HD uint32_t spread_sign(uint32_t x) {
+#ifdef __CUDA_ARCH__
+    uint32_t d;
+    asm("prmt.b32 %0, %1, %1, %2;" : "=r"(d) : "r"(x), "n"(0x8888 | 0x1111 * BYTE));
+    return d;
+#else
+    return 0u - ((x >> (8 * BYTE + 7)) & 1u);
+#endif
+}
+
+// The 32 bits of a word as masks, M[k] = bit k: seven shifts and 32 byte
+// permutes.
+TDES_HD void spread_bits(uint32_t x, uint32_t (&M)[32]) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const uint32_t y = x << (7 - k);
+        M[k] = spread_sign<0>(y);
+        M[8 + k] = spread_sign<1>(y);
+        M[16 + k] = spread_sign<2>(y);
+        M[24 + k] = spread_sign<3>(y);
+    }
+}
+
+// The CTR blocks of a lane's 32 slots, as the bit-planes that transposing
+// them would give: slot s = 2j + h holds counter c + 64 j + 2 lane + h under
+// the big-endian nonce.  The nonce planes are uniform; the counter planes are
+// a bitsliced addition of c + 2 lane and the slot's own bits (h at bit 0, j
+// at bits 6..9, constant patterns over the 32 slots) with the carry rippled
+// up.  About 180 logic operations where building the 64 words and transposing
+// them takes about 580.
+TDES_HD void counter_planes(uint32_t nonce, uint32_t c, uint32_t lane, uint32_t (&A0)[32],
+                            uint32_t (&A1)[32]) {
+    const uint32_t slot[5] = {0xAAAAAAAAu, 0xCCCCCCCCu, 0xF0F0F0F0u, 0xFF00FF00u, 0xFFFF0000u};
+    uint32_t M[32];
+    spread_bits(nonce, M);
+#pragma unroll
+    for (int k = 0; k < 32; ++k) A0[8 * (3 - k / 8) + k % 8] = M[k];
+    spread_bits(c + 2 * lane, M);
+    uint32_t carry = M[0] & slot[0];
+    A1[24] = M[0] ^ slot[0];
+#pragma unroll
+    for (int k = 1; k < 32; ++k) {
+        const int w = 8 * (3 - k / 8) + k % 8;  // counter bit k in the little-endian word
+        if (k >= 6 && k < 10) {
+            A1[w] = lop3<0x96>(M[k], slot[k - 5], carry);
+            carry = lop3<0xe8>(M[k], slot[k - 5], carry);
+        } else {
+            A1[w] = M[k] ^ carry;
+            carry &= M[k];
+        }
+    }
+}
+
 // 32 blocks: A0[s], A1[s] are the first and second little-endian 32-bit
 // words of block s on entry and of its result on return.
+// tdes_process32_planes takes bit-planes (A0[c] bit s = bit c of slot s's word).
 template <int STAGES = 3>
-TDES_HD void tdes_process32(uint32_t (&A0)[32], uint32_t (&A1)[32], const uint32_t* __restrict__ tab) {
-    transpose32(A0);
-    transpose32(A1);
+TDES_HD void tdes_process32_planes(uint32_t (&A0)[32], uint32_t (&A1)[32],
+                                   const uint32_t* __restrict__ tab) {
     uint32_t Lh[32], Rh[32];
     tdes_ip(A0, A1, Lh, Rh);
     tdes_rounds<STAGES>(Lh, Rh, tab);
     tdes_fp(Lh, Rh, A0, A1);
     transpose32(A0);
     transpose32(A1);
+}
+
+template <int STAGES = 3>
+TDES_HD void tdes_process32(uint32_t (&A0)[32], uint32_t (&A1)[32], const uint32_t* __restrict__ tab) {
+    transpose32(A0);
+    transpose32(A1);
+    tdes_process32_planes<STAGES>(A0, A1, tab);
 }
 
 TDES_HD void tdes_process32_rt(uint32_t (&A0)[32], uint32_t (&A1)[32],

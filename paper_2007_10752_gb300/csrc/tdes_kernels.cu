@@ -252,7 +252,8 @@ cudaError_t launch_ecb(const uint32_t* tab, int stages, const void* in, void* ou
 
 // ------------------------------------------------------------------- CTR
 // Keystream block i = E(nonce || ctr0 + i); the counter blocks are built in
-// registers.  The data tile the keystream is XORed into is copied into the
+// registers, directly as bit-planes (counter_planes: 3% fewer logic operations
+// a tile; 40 MB 118.8 -> 117.0 us).  The data tile the keystream is XORed into is copied into the
 // warp's 8 KiB of shared memory with cp.async before the rounds start, so
 // its memory latency hides behind them.
 template <bool VEC, int STAGES>
@@ -272,7 +273,6 @@ tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr
     // Tile indices fit 32 bits: the host caps a call below 2^31 tiles.
     using Idx = typename std::conditional<VEC, uint64_t, uint32_t>::type;
     const Idx ntiles = (Idx)((nblocks + kTileBlocks - 1) / kTileBlocks);
-    const uint32_t nw = bswap32(nonce);
     for (Idx t = (Idx)blockIdx.x * warps + (threadIdx.x >> 5); t < ntiles;
          t += (Idx)gridDim.x * warps) {
         const uint64_t b0 = (uint64_t)t * kTileBlocks;
@@ -284,15 +284,22 @@ tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr
             cp_async_commit();
         }
         uint32_t A0[32], A1[32];
+        if constexpr (VEC || STAGES == 1) {
+            counter_planes(nonce, ctr0 + (uint32_t)b0, lane, A0, A1);
+        } else {  // the 8-byte-aligned EDE3 variant would spill: words, transposed
+            const uint32_t nw = bswap32(nonce);
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
+            for (int j = 0; j < 16; ++j)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const uint32_t b = (uint32_t)b0 + 2u * (32u * j + lane) + h;
-                A0[2 * j + h] = nw;
-                A1[2 * j + h] = bswap32(ctr0 + b);
-            }
-        tdes_process32<STAGES>(A0, A1, tab);
+                for (int h = 0; h < 2; ++h) {
+                    const uint32_t b = (uint32_t)b0 + 2u * (32u * j + lane) + h;
+                    A0[2 * j + h] = nw;
+                    A1[2 * j + h] = bswap32(ctr0 + b);
+                }
+            transpose32(A0);
+            transpose32(A1);
+        }
+        tdes_process32_planes<STAGES>(A0, A1, tab);
         if (full) {
             cp_async_wait_all();
             uint4* q = reinterpret_cast<uint4*>(out) + (b0 >> 1) + lane;
