@@ -120,17 +120,17 @@ bool gpu_addressable(const void* p) {
     }
 }
 
-// Small inputs: one warp per CTA so the few tiles spread over many SMs.
-// Large inputs: kWideWarps warps per CTA, a grid of every resident CTA,
-// each warp striding over tiles.
+// Small inputs (a tile for each SM sub-partition at most): one warp per CTA so
+// the few tiles spread over many SMs.
+// Large inputs: kWideWarps warps per CTA, a grid of every resident CTA (also
+// where fewer would hold the tiles: every SM then gets the same number of
+// warps), each warp striding over tiles.
 Geometry geometry_for(uint64_t ntiles, int kernel_id, int device) {
     const DeviceInfo* d = device_info(device);
     const int sms = d ? d->sms : 1;
     const int per_sm = d ? d->ctas_per_sm[kernel_id] : 1;
-    if (ntiles <= (uint64_t)sms * kWideWarps) return {(int)(ntiles ? ntiles : 1), 32};
-    const uint64_t need = (ntiles + kWideWarps - 1) / kWideWarps;
-    const uint64_t full = (uint64_t)sms * per_sm;
-    return {(int)(need < full ? need : full), 32 * kWideWarps};
+    if (ntiles <= 4ull * sms) return {(int)(ntiles ? ntiles : 1), 32, sms};
+    return {sms * per_sm, 32 * kWideWarps, sms};
 }
 
 }  // namespace tdes
@@ -249,7 +249,7 @@ static int ecb(const tdes_ks_t* ks, int dir, const void* in, void* out, size_t n
     } else {
         const uint64_t ntiles = (nblocks + tdes::kTileBlocks - 1) / tdes::kTileBlocks;
         const tdes::Geometry g = tdes::geometry_for(ntiles, tdes::kEcb, ks->device);
-        e = tdes::launch_ecb(ks->tab[dir], ks->stages, in, out, nblocks, aligned16(in, out), g, s);
+        e = tdes::launch_ecb(ks->tab[dir], ks->chunk[dir], ks->stages, in, out, nblocks, aligned16(in, out), g, s);
     }
     return e == cudaSuccess ? TDES_OK : cuda_fail(e, "ECB kernel launch");
 }
@@ -280,7 +280,7 @@ int tdes_ctr_crypt(const tdes_ks_t* ks, uint32_t nonce, uint32_t ctr0, const voi
     } else {
         const uint64_t ntiles = (nblocks + tdes::kTileBlocks - 1) / tdes::kTileBlocks;
         const tdes::Geometry g = tdes::geometry_for(ntiles, tdes::kCtr, ks->device);
-        e = tdes::launch_ctr(ks->tab[0], ks->stages, nonce, ctr0, in, out, nblocks,
+        e = tdes::launch_ctr(ks->tab[0], ks->chunk[0], ks->stages, nonce, ctr0, in, out, nblocks,
                              aligned16(in, out), g, s);
     }
     return e == cudaSuccess ? TDES_OK : cuda_fail(e, "CTR kernel launch");
@@ -309,7 +309,7 @@ int tdes_cbc_decrypt(const tdes_ks_t* ks, uint64_t iv, const void* in, void* out
     }
     if (e == cudaSuccess) {
         const tdes::Geometry g = tdes::geometry_for(ntiles, tdes::kCbcDec, ks->device);
-        e = tdes::launch_cbc_dec(ks->tab[1], ks->stages, iv, in, out, nblocks, halo,
+        e = tdes::launch_cbc_dec(ks->tab[1], ks->chunk[1], ks->stages, iv, in, out, nblocks, halo,
                                  aligned16(in, out), g, s);
     }
     if (halo != nullptr) {
@@ -383,7 +383,7 @@ int tdes_ecb_crypt_host(const tdes_ks_t* ks, int decrypt, const void* host_in, v
         if (e == cudaSuccess) e = cudaStreamWaitEvent(scomp, ev_in[b], 0);
         if (e == cudaSuccess) {
             const tdes::Geometry g = tdes::geometry_for(ntiles, tdes::kEcb, ks->device);
-            e = tdes::launch_ecb(ks->tab[decrypt ? 1 : 0], ks->stages, buf, buf, nblocks, true,
+            e = tdes::launch_ecb(ks->tab[decrypt ? 1 : 0], ks->chunk[decrypt ? 1 : 0], ks->stages, buf, buf, nblocks, true,
                                  g, scomp);
         }
         if (e == cudaSuccess) e = cudaEventRecord(ev_k[b], scomp);

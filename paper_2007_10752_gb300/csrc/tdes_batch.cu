@@ -863,17 +863,19 @@ cudaError_t enqueue_direct(const std::vector<DirectMsg>& direct, const tdes_keyt
     for (const DirectMsg& m : direct) {
         const uint32_t dir = (m.mode == TDES_MODE_ECB_DECRYPT || m.mode == TDES_MODE_CBC_DECRYPT);
         const uint32_t* tab = kt->tabs + ((uint64_t)m.key * 2 + dir) * TDES_TABLE_WORDS;
+        const uint8_t* chunks =
+            kt->chunks + (uint64_t)m.key * kPerKeyChunks + TDES_SUBKEY_WORDS * dir;
         const bool vec16 = ((reinterpret_cast<uintptr_t>(m.in) | reinterpret_cast<uintptr_t>(m.out)) &
                             15u) == 0;
         const uint64_t ntiles = (m.nblocks + kTileBlocks - 1) / kTileBlocks;
         if (m.mode == TDES_MODE_CTR) {
-            e = launch_ctr(tab, m.stages, (uint32_t)(m.iv >> 32), (uint32_t)m.iv, m.in, m.out,
+            e = launch_ctr(tab, chunks, m.stages, (uint32_t)(m.iv >> 32), (uint32_t)m.iv, m.in, m.out,
                            m.nblocks, vec16, geometry_for(ntiles, kCtr, device), s);
         } else if (m.mode == TDES_MODE_CBC_DECRYPT) {
-            e = launch_cbc_dec(tab, m.stages, m.iv, m.in, m.out, m.nblocks, nullptr, vec16,
+            e = launch_cbc_dec(tab, chunks, m.stages, m.iv, m.in, m.out, m.nblocks, nullptr, vec16,
                                geometry_for(ntiles, kCbcDec, device), s);
         } else {
-            e = launch_ecb(tab, m.stages, m.in, m.out, m.nblocks, vec16,
+            e = launch_ecb(tab, chunks, m.stages, m.in, m.out, m.nblocks, vec16,
                            geometry_for(ntiles, kEcb, device), s);
         }
         if (e != cudaSuccess) return e;

@@ -41,24 +41,34 @@ struct Keys24 {
 struct Geometry {
     int grid;
     int threads;
+    int sms;
+};
+
+// The blocks of a call that run one per thread after the kernel's tiles: n of
+// them, right after the tiles' blocks; keys is the call's scalar round-key
+// groups on the device.
+struct Tail {
+    const uint32_t* keys;
+    uint32_t n;
 };
 Geometry geometry_for(uint64_t ntiles, int kernel_id, int device);
 
 enum KernelId { kEcb = 0, kCtr = 1, kCbcDec = 2, kNumKernels = 3 };
 
 // `stages` (1 or 3) selects the single-DES or the EDE3 kernels; the tables
-// passed must have been built for the same number of stages.
+// passed must have been built for the same number of stages.  chunks: the
+// scalar round-key groups of the same key and direction, on the device.
 cudaError_t launch_keysched(const Keys24& keys, int stages, uint32_t* tab_enc, uint32_t* tab_dec,
                             uint8_t* chunk_enc, uint8_t* chunk_dec, cudaStream_t s);
-cudaError_t launch_ecb(const uint32_t* tab, int stages, const void* in, void* out,
-                       uint64_t nblocks, bool vec16, Geometry g, cudaStream_t s);
-cudaError_t launch_ctr(const uint32_t* tab_enc, int stages, uint32_t nonce, uint32_t ctr0,
-                       const void* in, void* out, uint64_t nblocks, bool vec16, Geometry g,
-                       cudaStream_t s);
+cudaError_t launch_ecb(const uint32_t* tab, const uint8_t* chunks, int stages, const void* in,
+                       void* out, uint64_t nblocks, bool vec16, Geometry g, cudaStream_t s);
+cudaError_t launch_ctr(const uint32_t* tab_enc, const uint8_t* chunks, int stages, uint32_t nonce,
+                       uint32_t ctr0, const void* in, void* out, uint64_t nblocks, bool vec16,
+                       Geometry g, cudaStream_t s);
 cudaError_t launch_cbc_halo(const void* in, uint64_t* halo, uint64_t nblocks, cudaStream_t s);
-cudaError_t launch_cbc_dec(const uint32_t* tab_dec, int stages, uint64_t iv, const void* in,
-                           void* out, uint64_t nblocks, const uint64_t* halo, bool vec16,
-                           Geometry g, cudaStream_t s);
+cudaError_t launch_cbc_dec(const uint32_t* tab_dec, const uint8_t* chunks, int stages, uint64_t iv,
+                           const void* in, void* out, uint64_t nblocks, const uint64_t* halo,
+                           bool vec16, Geometry g, cudaStream_t s);
 cudaError_t launch_cbc_enc(const uint8_t* chunk_enc, int stages, uint64_t iv, const void* in,
                            void* out, uint64_t nblocks, cudaStream_t s);
 

@@ -14,6 +14,7 @@
 
 #include "tdes_internal.h"
 #include "tdes_keysched.cuh"
+#include "tdes_lanes.cuh"
 #include "tdes_scalar.cuh"
 
 namespace tdes {
@@ -125,6 +126,62 @@ __device__ __forceinline__ void store_tile(uint8_t* base, uint64_t b0, uint64_t 
 
 __device__ __forceinline__ uint32_t bswap32(uint32_t x) { return __byte_perm(x, 0u, 0x0123); }
 
+// ------------------------------------------------ first tile of a warp, tail
+// Tile of a warp's first pass (the later ones follow a stride of all warps).
+// The passes run CTA by CTA within a rank, and a CTA ranks its warps by SM
+// sub-partition, the first CTA of an SM from sub-partition 0 and the second
+// from 2, so that a last pass with fewer tiles than warps loads every
+// sub-partition alike: a tile alone on one takes 17 us, four together 46 us.
+// (Consecutive tiles per CTA put the 84 last tiles of 1300 on 11 SMs: 50.6
+// against 35.4 us.)  %warpid is only a hint: any values give each warp a rank
+// of its own.  publish_rank before a barrier, first_tile after it.
+__device__ __forceinline__ void publish_rank(uint32_t* order) {
+    uint32_t slot;
+    asm("mov.u32 %0, %%warpid;" : "=r"(slot));
+    if ((threadIdx.x & 31u) == 0)
+        order[threadIdx.x >> 5] =
+            8u * ((slot & 4u) | ((slot ^ (slot >> 2 & 2u)) & 3u)) + (threadIdx.x >> 5);
+}
+__device__ __forceinline__ uint32_t first_tile(const uint32_t* order) {
+    const uint32_t warps = blockDim.x >> 5, mine = order[threadIdx.x >> 5];
+    uint32_t rank = 0;
+    for (uint32_t w = 0; w < warps; ++w) rank += order[w] < mine;
+    return rank * gridDim.x + blockIdx.x;
+}
+
+// The blocks after the last whole round of tiles (tail_split): one block per
+// thread in every CTA, on the per-lane tables of tdes_lanes.cuh in the place
+// of the tile buffers.  A tile takes a sub-partition 7 us (next to others) to
+// 17 us (alone), however few tiles the last round has; the tail takes 2 us
+// and 4 us per 100 tiles.
+__device__ const uint32_t kTailSP[8][64] = TDES_SP_INIT;
+
+template <int MODE>
+__device__ __noinline__ void scalar_tail(Tail tail, uint64_t first, uint64_t iv, const uint8_t* in,
+                                         uint8_t* out, uint32_t* __restrict__ keys,
+                                         uint8_t* __restrict__ tab) {
+    const uint32_t share = ((tail.n + gridDim.x - 1) / gridDim.x + 31u) / 32u * 32u;
+    const uint32_t b0 = blockIdx.x * share;
+    if (b0 >= tail.n) return;
+    __syncthreads();  // every warp has left its tile buffer and the round constants
+    lane_tables(tab, &kTailSP[0][0]);
+    if (threadIdx.x < TDES_SUBKEY_WORDS / 4) keys[threadIdx.x] = __ldg(tail.keys + threadIdx.x);
+    __syncthreads();
+    const uint32_t end = min(b0 + share, tail.n), lane4 = (threadIdx.x & 31u) * 4u;
+    const uint64_t* p = reinterpret_cast<const uint64_t*>(in) + first;
+    uint64_t* q = reinterpret_cast<uint64_t*>(out) + first;
+    for (uint32_t b = b0 + threadIdx.x; b < end; b += blockDim.x) {
+        uint64_t x = bswap64(p[b]), other = 0;
+        if (MODE == kSmallCtr) {
+            other = x;
+            x = (iv & 0xFFFFFFFF00000000ull) | (uint32_t)((uint32_t)iv + (uint32_t)first + b);
+        } else if (MODE == kSmallCbcDec) {
+            other = bswap64(p[(int64_t)b - 1]);  // a tail never starts at block 0
+        }
+        q[b] = bswap64(lane_block<48>(x, keys, lane4, tab) ^ other);
+    }
+}
+
 // ------------------------------------------------------------------- ECB
 // Full tiles of 16-byte-aligned buffers are prefetched one tile ahead into the
 // warp's 8 KiB of shared memory with cp.async, so the next tile's memory
@@ -144,10 +201,12 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 template <bool VEC, int STAGES>
 __global__ void __launch_bounds__(256, 2)
 tdes_ecb_kernel(const uint32_t* __restrict__ table, const uint8_t* in, uint8_t* out,
-                uint64_t nblocks) {
+                uint64_t nblocks, Tail tail) {
     __shared__ __align__(16) uint32_t tab[table_words<STAGES>()];
     extern __shared__ __align__(16) uint4 ecb_data[];  // kCtrWarpBytes per warp (VEC only)
+    __shared__ uint32_t order[kWideWarps];
     stage_table<STAGES>(tab, table);
+    publish_rank(order);
     __syncthreads();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warps = blockDim.x >> 5;
@@ -156,7 +215,7 @@ tdes_ecb_kernel(const uint32_t* __restrict__ table, const uint8_t* in, uint8_t* 
     const uint32_t ntiles = (uint32_t)((nblocks + kTileBlocks - 1) / kTileBlocks);
     const uint32_t nfull = (uint32_t)(nblocks / kTileBlocks);  // tiles [0, nfull) are full
     const uint32_t stride = gridDim.x * warps;
-    uint32_t t = blockIdx.x * warps + (threadIdx.x >> 5);
+    uint32_t t = first_tile(order);
     if (VEC && t < nfull) {
         const uint4* p = reinterpret_cast<const uint4*>(in) + (uint64_t)t * (kTileBlocks / 2) + lane;
 #pragma unroll
@@ -189,17 +248,21 @@ tdes_ecb_kernel(const uint32_t* __restrict__ table, const uint8_t* in, uint8_t* 
         tdes_process32<STAGES>(A0, A1, tab);
         store_tile<VEC>(out, (uint64_t)t * kTileBlocks, nblocks, lane, A0, A1);
     }
+    if constexpr (VEC && STAGES == 3)
+        if (tail.n)
+            scalar_tail<kSmallEcb>(tail, nblocks, 0, in, out, tab,
+                                   reinterpret_cast<uint8_t*>(ecb_data));
 }
 
 // The kernels that stage data tiles take up to kWideWarps x 8 KiB of dynamic
 // shared memory, above the default limit: raise it once per device.
 template <bool VEC, int STAGES>
 __global__ void tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr0,
-                                const uint8_t* in, uint8_t* out, uint64_t nblocks);
+                                const uint8_t* in, uint8_t* out, uint64_t nblocks, Tail tail);
 template <bool VEC, int STAGES>
 __global__ void tdes_cbc_dec_kernel(const uint32_t* __restrict__ table, uint64_t iv,
                                     const uint8_t* in, uint8_t* out, uint64_t nblocks,
-                                    const uint64_t* __restrict__ halo);
+                                    const uint64_t* __restrict__ halo, Tail tail);
 
 static std::atomic<bool> dyn_smem_ready[64];
 
@@ -227,26 +290,45 @@ static cudaError_t ensure_dyn_smem() {
     return cudaSuccess;
 }
 
+// Splits a call: the blocks that run as tiles, and the tail.  A sub-partition
+// takes whole tiles, so the time of a call rises in steps of one tile for each
+// of them (608 tiles); when few blocks lie past the last step they run as the
+// tail instead: up to 320 tiles' worth where the tiles fill whole passes (the
+// step there costs a lone tile's 17 us), else up to 128 (7 us).
+static uint64_t tail_split(int stages, bool vec16, Geometry g, const uint8_t* chunks,
+                           uint64_t nblocks, Tail* tail) {
+    *tail = Tail{nullptr, 0};
+    if (stages != 3 || !vec16 || chunks == nullptr || g.threads != 32 * kWideWarps) return nblocks;
+    const uint64_t step = 4ull * g.sms * kTileBlocks, steps = nblocks / step;
+    const uint64_t rest = nblocks - steps * step;
+    if (steps == 0 || rest > (steps % 4 == 0 ? 320u : 128u) * (uint64_t)kTileBlocks) return nblocks;
+    tail->keys = reinterpret_cast<const uint32_t*>(chunks);
+    tail->n = (uint32_t)rest;
+    return steps * step;
+}
+
 template <int STAGES>
 static void ecb_launch(const uint32_t* tab, const void* in, void* out, uint64_t nblocks,
-                       bool vec16, Geometry g, cudaStream_t s) {
+                       bool vec16, Geometry g, Tail tail, cudaStream_t s) {
     if (vec16)
         tdes_ecb_kernel<true, STAGES>
             <<<g.grid, g.threads, (size_t)(g.threads / 32) * kCtrWarpBytes, s>>>(
-                tab, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out), nblocks);
+                tab, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out), nblocks, tail);
     else
         tdes_ecb_kernel<false, STAGES><<<g.grid, g.threads, 0, s>>>(
-            tab, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out), nblocks);
+            tab, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out), nblocks, tail);
 }
 
-cudaError_t launch_ecb(const uint32_t* tab, int stages, const void* in, void* out,
-                       uint64_t nblocks, bool vec16, Geometry g, cudaStream_t s) {
+cudaError_t launch_ecb(const uint32_t* tab, const uint8_t* chunks, int stages, const void* in,
+                       void* out, uint64_t nblocks, bool vec16, Geometry g, cudaStream_t s) {
     cudaError_t e = ensure_dyn_smem();
     if (e != cudaSuccess) return e;
+    Tail tail;
+    nblocks = tail_split(stages, vec16, g, chunks, nblocks, &tail);
     if (stages == 1)
-        ecb_launch<1>(tab, in, out, nblocks, vec16, g, s);
+        ecb_launch<1>(tab, in, out, nblocks, vec16, g, tail, s);
     else
-        ecb_launch<3>(tab, in, out, nblocks, vec16, g, s);
+        ecb_launch<3>(tab, in, out, nblocks, vec16, g, tail, s);
     return cudaGetLastError();
 }
 
@@ -259,10 +341,12 @@ cudaError_t launch_ecb(const uint32_t* tab, int stages, const void* in, void* ou
 template <bool VEC, int STAGES>
 __global__ void __launch_bounds__(256, 2)
 tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr0,
-                const uint8_t* in, uint8_t* out, uint64_t nblocks) {
+                const uint8_t* in, uint8_t* out, uint64_t nblocks, Tail tail) {
     __shared__ __align__(16) uint32_t tab[table_words<STAGES>()];
     extern __shared__ __align__(16) uint4 ctr_data[];  // kCtrWarpBytes per warp
+    __shared__ uint32_t order[kWideWarps];
     stage_table<STAGES>(tab, table);
+    publish_rank(order);
     __syncthreads();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warps = blockDim.x >> 5;
@@ -273,8 +357,7 @@ tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr
     // Tile indices fit 32 bits: the host caps a call below 2^31 tiles.
     using Idx = typename std::conditional<VEC, uint64_t, uint32_t>::type;
     const Idx ntiles = (Idx)((nblocks + kTileBlocks - 1) / kTileBlocks);
-    for (Idx t = (Idx)blockIdx.x * warps + (threadIdx.x >> 5); t < ntiles;
-         t += (Idx)gridDim.x * warps) {
+    for (Idx t = first_tile(order); t < ntiles; t += (Idx)gridDim.x * warps) {
         const uint64_t b0 = (uint64_t)t * kTileBlocks;
         const bool full = VEC && b0 + kTileBlocks <= nblocks;
         if (full) {  // each lane copies, and later reads back, only its own 16 x 16 bytes
@@ -338,31 +421,38 @@ tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr
                 }
         }
     }
+    if constexpr (VEC && STAGES == 3)
+        if (tail.n)
+            scalar_tail<kSmallCtr>(tail, nblocks, (uint64_t)nonce << 32 | ctr0, in, out, tab,
+                                   reinterpret_cast<uint8_t*>(ctr_data));
 }
 
 template <int STAGES>
 static void ctr_launch(const uint32_t* tab_enc, uint32_t nonce, uint32_t ctr0, const void* in,
-                       void* out, uint64_t nblocks, bool vec16, Geometry g, cudaStream_t s) {
+                       void* out, uint64_t nblocks, bool vec16, Geometry g, Tail tail,
+                       cudaStream_t s) {
     const size_t dyn = (size_t)(g.threads / 32) * kCtrWarpBytes;
     if (vec16)
         tdes_ctr_kernel<true, STAGES><<<g.grid, g.threads, dyn, s>>>(
             tab_enc, nonce, ctr0, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out),
-            nblocks);
+            nblocks, tail);
     else
         tdes_ctr_kernel<false, STAGES><<<g.grid, g.threads, dyn, s>>>(
             tab_enc, nonce, ctr0, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out),
-            nblocks);
+            nblocks, tail);
 }
 
-cudaError_t launch_ctr(const uint32_t* tab_enc, int stages, uint32_t nonce, uint32_t ctr0,
-                       const void* in, void* out, uint64_t nblocks, bool vec16, Geometry g,
-                       cudaStream_t s) {
+cudaError_t launch_ctr(const uint32_t* tab_enc, const uint8_t* chunks, int stages, uint32_t nonce,
+                       uint32_t ctr0, const void* in, void* out, uint64_t nblocks, bool vec16,
+                       Geometry g, cudaStream_t s) {
     cudaError_t e = ensure_dyn_smem();
     if (e != cudaSuccess) return e;
+    Tail tail;
+    nblocks = tail_split(stages, vec16, g, chunks, nblocks, &tail);
     if (stages == 1)
-        ctr_launch<1>(tab_enc, nonce, ctr0, in, out, nblocks, vec16, g, s);
+        ctr_launch<1>(tab_enc, nonce, ctr0, in, out, nblocks, vec16, g, tail, s);
     else
-        ctr_launch<3>(tab_enc, nonce, ctr0, in, out, nblocks, vec16, g, s);
+        ctr_launch<3>(tab_enc, nonce, ctr0, in, out, nblocks, vec16, g, tail, s);
     return cudaGetLastError();
 }
 
@@ -390,10 +480,13 @@ cudaError_t launch_cbc_halo(const void* in, uint64_t* halo, uint64_t nblocks, cu
 template <bool VEC, int STAGES>
 __global__ void __launch_bounds__(256, 2)
 tdes_cbc_dec_kernel(const uint32_t* __restrict__ table, uint64_t iv, const uint8_t* in,
-                    uint8_t* out, uint64_t nblocks, const uint64_t* __restrict__ halo) {
+                    uint8_t* out, uint64_t nblocks, const uint64_t* __restrict__ halo,
+                    Tail tail) {
     __shared__ __align__(16) uint32_t tab[table_words<STAGES>()];
     extern __shared__ __align__(16) uint4 cbc_data[];  // kCtrWarpBytes per warp (VEC only)
+    __shared__ uint32_t order[kWideWarps];
     stage_table<STAGES>(tab, table);
+    publish_rank(order);
     __syncthreads();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warps = blockDim.x >> 5;
@@ -404,7 +497,7 @@ tdes_cbc_dec_kernel(const uint32_t* __restrict__ table, uint64_t iv, const uint8
     const uint32_t stride = gridDim.x * warps;
     const uint2 ivw = make_uint2(bswap32((uint32_t)(iv >> 32)), bswap32((uint32_t)iv));
     const uint2* c = reinterpret_cast<const uint2*>(in);
-    uint32_t t = blockIdx.x * warps + (threadIdx.x >> 5);
+    uint32_t t = first_tile(order);
     if (VEC && t < nfull) {  // full tiles are prefetched one ahead, as in ECB
         const uint4* p = reinterpret_cast<const uint4*>(in) + (uint64_t)t * (kTileBlocks / 2) + lane;
 #pragma unroll
@@ -464,32 +557,38 @@ tdes_cbc_dec_kernel(const uint32_t* __restrict__ table, uint64_t iv, const uint8
         __syncwarp();
         store_tile<VEC>(out, b0, nblocks, lane, A0, A1);
     }
+    if constexpr (VEC && STAGES == 3)
+        if (tail.n)
+            scalar_tail<kSmallCbcDec>(tail, nblocks, iv, in, out, tab,
+                                      reinterpret_cast<uint8_t*>(cbc_data));
 }
 
 template <int STAGES>
 static void cbc_dec_launch(const uint32_t* tab_dec, uint64_t iv, const void* in, void* out,
                            uint64_t nblocks, const uint64_t* halo, bool vec16, Geometry g,
-                           cudaStream_t s) {
+                           Tail tail, cudaStream_t s) {
     if (vec16)
         tdes_cbc_dec_kernel<true, STAGES>
             <<<g.grid, g.threads, (size_t)(g.threads / 32) * kCtrWarpBytes, s>>>(
                 tab_dec, iv, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out),
-                nblocks, halo);
+                nblocks, halo, tail);
     else
         tdes_cbc_dec_kernel<false, STAGES><<<g.grid, g.threads, 0, s>>>(
             tab_dec, iv, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out), nblocks,
-            halo);
+            halo, tail);
 }
 
-cudaError_t launch_cbc_dec(const uint32_t* tab_dec, int stages, uint64_t iv, const void* in,
-                           void* out, uint64_t nblocks, const uint64_t* halo, bool vec16,
-                           Geometry g, cudaStream_t s) {
+cudaError_t launch_cbc_dec(const uint32_t* tab_dec, const uint8_t* chunks, int stages, uint64_t iv,
+                           const void* in, void* out, uint64_t nblocks, const uint64_t* halo,
+                           bool vec16, Geometry g, cudaStream_t s) {
     cudaError_t e = ensure_dyn_smem();
     if (e != cudaSuccess) return e;
+    Tail tail;  // in place a tail block's predecessor may be overwritten before it is read
+    nblocks = tail_split(stages, vec16, g, in == out ? nullptr : chunks, nblocks, &tail);
     if (stages == 1)
-        cbc_dec_launch<1>(tab_dec, iv, in, out, nblocks, halo, vec16, g, s);
+        cbc_dec_launch<1>(tab_dec, iv, in, out, nblocks, halo, vec16, g, tail, s);
     else
-        cbc_dec_launch<3>(tab_dec, iv, in, out, nblocks, halo, vec16, g, s);
+        cbc_dec_launch<3>(tab_dec, iv, in, out, nblocks, halo, vec16, g, tail, s);
     return cudaGetLastError();
 }
 
