@@ -61,34 +61,32 @@ TDES_HD void tdes_round_mixed(uint32_t (&T)[32], const uint32_t (&S)[32],
     const uint32_t x4 = S[7];
     const uint32_t x5 = S[8];
     const uint4 kc = *reinterpret_cast<const uint4*>(k + 8);
-    const uint32_t s1_0 = lop3<0x7e>(x5, x4, x0);
-    const uint32_t s1_1 = lop3<0xe8>(s1_0, x4, x1);
-    const uint32_t s1_2 = lop3<0x84>(x1, x5, x0);
-    const uint32_t s1_3 = lop3<0x17>(s1_2, x4, x1);
-    const uint32_t s1_4 = lop3<0xbd>(x5, x1, x0);
-    const uint32_t s1_5 = lop3<0x70>(s1_4, x4, x0);
-    const uint32_t s1_6 = lop3<0x93>(s1_3, s1_5, x3);
-    const uint32_t s1_7 = lop3<0x86>(s1_6, s1_3, s1_0);
-    const uint32_t s1_8 = lop3<0xe4>(s1_7, s1_6, x2);
-    T[17] = lop3<0x69>(T[17], s1_8, kc.w);
-    const uint32_t s1_9 = lop3<0x18>(s1_8, s1_5, x1);
-    const uint32_t s1_10 = lop3<0x6b>(s1_9, x4, x0);
-    const uint32_t s1_11 = lop3<0x69>(s1_10, x1, x2);
-    const uint32_t s1_12 = lop3<0x6d>(s1_11, s1_2, s1_5);
-    const uint32_t s1_13 = lop3<0x93>(s1_1, s1_12, x3);
+    const uint32_t s1_0 = lop3<0xb1>(x4, x1, x0);
+    const uint32_t s1_1 = lop3<0x43>(x5, s1_0, x1);
+    const uint32_t s1_2 = lop3<0xbd>(x1, x5, x0);
+    const uint32_t s1_3 = lop3<0x84>(s1_2, x4, x0);
+    const uint32_t s1_4 = lop3<0x67>(s1_1, s1_0, x0);
+    const uint32_t s1_5 = lop3<0x16>(s1_4, x4, x1);
+    const uint32_t s1_6 = lop3<0x6f>(s1_4, s1_5, x5);
+    const uint32_t s1_7 = lop3<0xa6>(s1_5, x3, x2);
+    const uint32_t s1_8 = lop3<0x67>(s1_2, s1_7, s1_3);
+    const uint32_t s1_9 = lop3<0x95>(s1_6, s1_8, x3);
+    T[17] = lop3<0x96>(T[17], s1_9, kc.w);
+    const uint32_t s1_10 = lop3<0xb6>(s1_9, x5, x0);
+    const uint32_t s1_11 = lop3<0x58>(s1_5, s1_3, x2);
+    const uint32_t s1_12 = lop3<0x9a>(s1_10, s1_4, x4);
+    const uint32_t s1_13 = lop3<0x69>(s1_12, s1_1, s1_7);
     T[12] = lop3<0x96>(T[12], s1_13, kc.x);
-    const uint32_t s1_14 = lop3<0x56>(s1_13, s1_4, x4);
-    const uint32_t s1_15 = lop3<0x2e>(s1_13, s1_11, s1_8);
-    const uint32_t s1_16 = lop3<0x4a>(s1_15, s1_5, x5);
-    const uint32_t s1_17 = lop3<0xa9>(s1_14, s1_16, s1_8);
-    const uint32_t s1_18 = lop3<0x96>(s1_17, s1_13, x1);
-    T[27] = lop3<0x96>(T[27], s1_18, kc.y);
-    const uint32_t s1_19 = lop3<0x92>(s1_6, s1_16, s1_1);
-    const uint32_t s1_20 = lop3<0x13>(s1_8, s1_19, s1_13);
-    const uint32_t s1_21 = lop3<0x5e>(s1_20, s1_16, s1_10);
-    const uint32_t s1_22 = lop3<0x49>(s1_18, s1_14, s1_6);
-    const uint32_t s1_23 = lop3<0x87>(s1_21, s1_22, x0);
-    T[1] = lop3<0x96>(T[1], s1_23, kc.z);
+    const uint32_t s1_14 = lop3<0x53>(s1_10, s1_13, x0);
+    const uint32_t s1_15 = lop3<0xe9>(s1_14, s1_13, s1_2);
+    const uint32_t s1_16 = lop3<0xe5>(s1_14, s1_13, x5);
+    const uint32_t s1_17 = lop3<0x0c>(s1_13, s1_2, s1_0);
+    const uint32_t s1_18 = lop3<0x6c>(s1_16, s1_17, x4);
+    const uint32_t s1_19 = lop3<0x69>(s1_18, s1_9, x1);
+    T[27] = lop3<0x69>(T[27], s1_19, kc.y);
+    const uint32_t s1_20 = lop3<0x8d>(s1_15, s1_11, s1_9);
+    const uint32_t s1_21 = lop3<0x49>(s1_12, s1_16, s1_20);
+    T[1] = lop3<0x96>(T[1], s1_21, kc.z);
     }
     {  // S-box 3
     const uint4 kd = *reinterpret_cast<const uint4*>(k + 20);
@@ -99,33 +97,32 @@ TDES_HD void tdes_round_mixed(uint32_t (&T)[32], const uint32_t (&S)[32],
     const uint32_t x4 = S[11];
     const uint32_t x5 = S[12];
     const uint4 kc = *reinterpret_cast<const uint4*>(k + 16);
-    const uint32_t s2_0 = lop3<0xac>(x4, x3, x2);
-    const uint32_t s2_1 = lop3<0x69>(s2_0, x5, x1);
-    const uint32_t s2_2 = lop3<0x9e>(s2_1, x2, x1);
-    const uint32_t s2_3 = lop3<0xf1>(x4, x2, x1);
-    const uint32_t s2_4 = lop3<0xe4>(s2_2, s2_3, x5);
-    const uint32_t s2_5 = lop3<0x18>(s2_2, s2_1, x0);
-    const uint32_t s2_6 = lop3<0x42>(s2_4, s2_5, x1);
-    const uint32_t s2_7 = lop3<0x43>(s2_4, x4, x3);
-    const uint32_t s2_8 = lop3<0x39>(s2_7, s2_1, x0);
-    T[5] = lop3<0x96>(T[5], s2_8, kc.w);
-    const uint32_t s2_9 = lop3<0xe4>(s2_4, s2_8, s2_0);
-    const uint32_t s2_10 = lop3<0x6b>(s2_9, x2, x0);
-    const uint32_t s2_11 = lop3<0x96>(x4, s2_10, x5);
-    const uint32_t s2_12 = lop3<0xc6>(s2_6, s2_11, x3);
-    T[23] = lop3<0x96>(T[23], s2_12, kc.x);
-    const uint32_t s2_13 = lop3<0x67>(s2_3, s2_1, x0);
-    const uint32_t s2_14 = lop3<0xa6>(s2_0, s2_13, x1);
-    const uint32_t s2_15 = lop3<0x24>(s2_14, s2_1, x4);
-    const uint32_t s2_16 = lop3<0xda>(s2_13, s2_5, x2);
-    const uint32_t s2_17 = lop3<0x39>(s2_15, s2_16, x3);
-    T[15] = lop3<0x96>(T[15], s2_17, kc.y);
-    const uint32_t s2_18 = lop3<0xd6>(s2_11, s2_3, x3);
-    const uint32_t s2_19 = lop3<0xa6>(s2_12, s2_18, s2_13);
-    const uint32_t s2_20 = lop3<0x96>(s2_17, s2_14, s2_2);
-    const uint32_t s2_21 = lop3<0xc2>(s2_20, s2_18, x5);
-    const uint32_t s2_22 = lop3<0xb4>(s2_19, x1, s2_21);
-    T[29] = lop3<0x96>(T[29], s2_22, kc.z);
+    const uint32_t s2_0 = lop3<0x3c>(x5, x3, x1);
+    const uint32_t s2_1 = lop3<0x86>(x5, x4, x2);
+    const uint32_t s2_2 = lop3<0xb1>(s2_1, s2_0, x4);
+    const uint32_t s2_3 = lop3<0x69>(x1, s2_2, x0);
+    const uint32_t s2_4 = lop3<0xde>(s2_1, s2_0, x1);
+    const uint32_t s2_5 = lop3<0xbe>(s2_4, x1, x0);
+    const uint32_t s2_6 = lop3<0x62>(s2_5, s2_3, x2);
+    const uint32_t s2_7 = lop3<0x87>(s2_6, s2_4, x3);
+    T[15] = lop3<0x69>(T[15], s2_7, kc.y);
+    const uint32_t s2_8 = lop3<0xf4>(s2_7, x5, x3);
+    const uint32_t s2_9 = lop3<0x37>(s2_8, s2_3, x0);
+    const uint32_t s2_10 = lop3<0x46>(s2_9, s2_6, x4);
+    const uint32_t s2_11 = lop3<0x72>(s2_10, s2_1, x5);
+    const uint32_t s2_12 = lop3<0x5e>(s2_11, s2_3, x3);
+    const uint32_t s2_13 = lop3<0xb6>(s2_8, x4, x1);
+    const uint32_t s2_14 = lop3<0xb5>(s2_11, s2_8, x0);
+    const uint32_t s2_15 = lop3<0x36>(s2_14, x1, s2_1);
+    const uint32_t s2_16 = lop3<0xd6>(s2_15, x0, x2);
+    const uint32_t s2_17 = lop3<0x69>(s2_16, x4, s2_0);
+    T[23] = lop3<0x69>(T[23], s2_17, kc.x);
+    const uint32_t s2_18 = lop3<0x25>(s2_17, s2_10, s2_9);
+    const uint32_t s2_19 = lop3<0x87>(s2_18, s2_12, x1);
+    T[29] = lop3<0x96>(T[29], s2_19, kc.z);
+    const uint32_t s2_20 = lop3<0xb3>(s2_19, s2_13, x5);
+    const uint32_t s2_21 = lop3<0xc6>(s2_20, s2_3, x0);
+    T[5] = lop3<0x96>(T[5], s2_21, kc.w);
     }
     {  // S-box 4
     const uint4 kd = *reinterpret_cast<const uint4*>(k + 28);
@@ -136,28 +133,26 @@ TDES_HD void tdes_round_mixed(uint32_t (&T)[32], const uint32_t (&S)[32],
     const uint32_t x4 = S[15];
     const uint32_t x5 = S[16];
     const uint4 kc = *reinterpret_cast<const uint4*>(k + 24);
-    const uint32_t s3_0 = lop3<0x56>(x4, x2, x0);
-    const uint32_t s3_1 = lop3<0x39>(s3_0, x3, x2);
-    const uint32_t s3_2 = lop3<0xf6>(x2, x1, x0);
-    const uint32_t s3_3 = lop3<0x4e>(s3_1, s3_2, x4);
-    const uint32_t s3_4 = lop3<0x94>(x3, s3_3, x1);
-    const uint32_t s3_5 = lop3<0x63>(s3_4, s3_1, x4);
-    const uint32_t s3_6 = lop3<0x78>(s3_4, s3_2, x4);
-    const uint32_t s3_7 = lop3<0x9c>(x4, s3_4, x1);
-    const uint32_t s3_8 = lop3<0xbd>(s3_7, s3_5, x2);
-    const uint32_t s3_9 = lop3<0x96>(s3_8, s3_2, x4);
-    const uint32_t s3_10 = lop3<0x5b>(s3_6, s3_9, x2);
-    const uint32_t s3_11 = lop3<0x93>(x1, s3_5, s3_10);
-    const uint32_t s3_12 = lop3<0x84>(s3_11, s3_9, x2);
-    const uint32_t s3_13 = lop3<0x39>(s3_12, s3_4, s3_0);
-    const uint32_t s3_14 = lop3<0x72>(s3_13, s3_11, x5);
-    T[25] = lop3<0x69>(T[25], s3_14, kc.x);
-    const uint32_t s3_15 = lop3<0x1b>(s3_13, s3_11, x5);
-    T[19] = lop3<0x69>(T[19], s3_15, kc.y);
-    const uint32_t s3_16 = lop3<0x27>(s3_9, s3_6, x5);
-    T[9] = lop3<0x69>(T[9], s3_16, kc.z);
-    const uint32_t s3_17 = lop3<0x4e>(s3_9, s3_6, x5);
-    T[0] = lop3<0x69>(T[0], s3_17, kc.w);
+    const uint32_t s3_0 = lop3<0x78>(x3, x2, x0);
+    const uint32_t s3_1 = lop3<0x87>(x4, x2, x1);
+    const uint32_t s3_2 = lop3<0x7c>(s3_1, x1, x0);
+    const uint32_t s3_3 = lop3<0x65>(s3_2, s3_0, x2);
+    const uint32_t s3_4 = lop3<0x96>(s3_3, s3_1, x0);
+    const uint32_t s3_5 = lop3<0x59>(s3_4, s3_1, x1);
+    const uint32_t s3_6 = lop3<0xd2>(s3_0, s3_5, s3_2);
+    const uint32_t s3_7 = lop3<0x84>(s3_6, s3_5, x0);
+    const uint32_t s3_8 = lop3<0x34>(s3_6, s3_4, x0);
+    const uint32_t s3_9 = lop3<0x1c>(s3_8, s3_4, x4);
+    const uint32_t s3_10 = lop3<0x1e>(s3_3, s3_8, s3_7);
+    const uint32_t s3_11 = lop3<0x1b>(s3_10, s3_4, x5);
+    T[0] = lop3<0x69>(T[0], s3_11, kc.w);
+    const uint32_t s3_12 = lop3<0x8d>(s3_10, s3_4, x5);
+    T[9] = lop3<0x69>(T[9], s3_12, kc.z);
+    const uint32_t s3_13 = lop3<0x96>(s3_10, s3_9, x3);
+    const uint32_t s3_14 = lop3<0x27>(s3_13, s3_6, x5);
+    T[25] = lop3<0x96>(T[25], s3_14, kc.x);
+    const uint32_t s3_15 = lop3<0xb1>(s3_13, s3_6, x5);
+    T[19] = lop3<0x96>(T[19], s3_15, kc.y);
     }
     {  // S-box 5
     const uint4 kd = *reinterpret_cast<const uint4*>(k + 36);
@@ -168,36 +163,35 @@ TDES_HD void tdes_round_mixed(uint32_t (&T)[32], const uint32_t (&S)[32],
     const uint32_t x4 = S[19];
     const uint32_t x5 = S[20];
     const uint4 kc = *reinterpret_cast<const uint4*>(k + 32);
-    const uint32_t s4_0 = lop3<0x71>(x5, x3, x0);
-    const uint32_t s4_1 = lop3<0x6e>(x5, s4_0, x2);
-    const uint32_t s4_2 = lop3<0xeb>(x0, s4_1, x3);
-    const uint32_t s4_3 = lop3<0x7d>(x4, s4_1, x2);
-    const uint32_t s4_4 = lop3<0xe6>(s4_2, x0, x4);
-    const uint32_t s4_5 = lop3<0x9e>(s4_4, x5, x2);
-    const uint32_t s4_6 = lop3<0x42>(s4_1, x5, x0);
-    const uint32_t s4_7 = lop3<0x94>(s4_3, x3, x0);
-    const uint32_t s4_8 = lop3<0xe3>(s4_7, s4_2, x5);
-    const uint32_t s4_9 = lop3<0xe4>(s4_8, s4_1, x4);
-    const uint32_t s4_10 = lop3<0x7a>(s4_9, x4, x1);
-    const uint32_t s4_11 = lop3<0x70>(s4_10, s4_7, x1);
-    T[24] = lop3<0x96>(T[24], s4_11, kc.z);
-    const uint32_t s4_12 = lop3<0x94>(s4_9, s4_7, s4_6);
-    const uint32_t s4_13 = lop3<0x90>(s4_9, s4_3, s4_5);
-    const uint32_t s4_14 = lop3<0xa9>(s4_13, s4_5, x3);
-    const uint32_t s4_15 = lop3<0x5b>(s4_14, s4_4, s4_3);
-    const uint32_t s4_16 = lop3<0x78>(s4_15, s4_2, x1);
-    T[13] = lop3<0x96>(T[13], s4_16, kc.y);
-    const uint32_t s4_17 = lop3<0xde>(s4_16, s4_15, x3);
-    const uint32_t s4_18 = lop3<0xf2>(s4_12, s4_11, s4_1);
-    const uint32_t s4_19 = lop3<0x95>(s4_13, s4_18, s4_11);
-    const uint32_t s4_20 = lop3<0xbc>(s4_19, s4_14, x1);
-    const uint32_t s4_21 = lop3<0x78>(s4_20, x1, x4);
-    const uint32_t s4_22 = lop3<0x63>(x5, s4_21, s4_17);
-    T[2] = lop3<0x96>(T[2], s4_22, kc.w);
-    const uint32_t s4_23 = lop3<0x28>(s4_22, s4_3, x4);
-    const uint32_t s4_24 = lop3<0x49>(s4_4, s4_23, s4_6);
-    const uint32_t s4_25 = lop3<0x9a>(x1, s4_24, s4_18);
-    T[7] = lop3<0x96>(T[7], s4_25, kc.x);
+    const uint32_t s4_0 = lop3<0x25>(x5, x3, x0);
+    const uint32_t s4_1 = lop3<0x68>(s4_0, x2, x0);
+    const uint32_t s4_2 = lop3<0x82>(s4_1, x4, x2);
+    const uint32_t s4_3 = lop3<0x4a>(s4_2, x0, x3);
+    const uint32_t s4_4 = lop3<0x49>(s4_2, x3, x0);
+    const uint32_t s4_5 = lop3<0x9a>(x4, s4_1, s4_4);
+    const uint32_t s4_6 = lop3<0xb9>(s4_4, x2, s4_0);
+    const uint32_t s4_7 = lop3<0x75>(s4_6, x3, x1);
+    const uint32_t s4_8 = lop3<0x34>(s4_5, s4_3, x0);
+    const uint32_t s4_9 = lop3<0xe9>(s4_8, x2, x5);
+    const uint32_t s4_10 = lop3<0x69>(s4_9, s4_3, s4_7);
+    T[13] = lop3<0x96>(T[13], s4_10, kc.y);
+    const uint32_t s4_11 = lop3<0x24>(s4_10, s4_7, x3);
+    const uint32_t s4_12 = lop3<0x7e>(s4_10, s4_5, x5);
+    const uint32_t s4_13 = lop3<0x5a>(s4_9, x5, x3);
+    const uint32_t s4_14 = lop3<0x9d>(s4_13, x4, x0);
+    const uint32_t s4_15 = lop3<0x82>(s4_14, s4_6, s4_7);
+    const uint32_t s4_16 = lop3<0x52>(s4_15, s4_4, x1);
+    T[24] = lop3<0x96>(T[24], s4_16, kc.z);
+    const uint32_t s4_17 = lop3<0x43>(s4_16, s4_15, s4_12);
+    const uint32_t s4_18 = lop3<0x2c>(s4_17, s4_13, s4_7);
+    const uint32_t s4_19 = lop3<0x8c>(s4_12, s4_11, x5);
+    const uint32_t s4_20 = lop3<0x96>(s4_19, s4_18, x1);
+    const uint32_t s4_21 = lop3<0xd2>(s4_20, x4, x1);
+    T[2] = lop3<0x96>(T[2], s4_21, kc.w);
+    const uint32_t s4_22 = lop3<0xb9>(x4, s4_21, s4_10);
+    const uint32_t s4_23 = lop3<0x14>(s4_22, s4_16, s4_8);
+    const uint32_t s4_24 = lop3<0xa6>(s4_23, s4_12, x1);
+    T[7] = lop3<0x69>(T[7], s4_24, kc.x);
     }
     {  // S-box 6
     const uint4 kd = *reinterpret_cast<const uint4*>(k + 44);
