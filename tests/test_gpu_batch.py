@@ -365,3 +365,37 @@ def test_large_messages_run_direct(cuda_lib):
     torch.cuda.synchronize()
     for i, (_, x, y) in enumerate(bufs):
         assert (y.cpu().numpy() == outs[i]).all(), f"message {i} graph replay"
+
+
+@pytest.mark.parametrize("lens", [[8 * 509] * 3, [8 * n for n in range(1, 90)] * 8, [8 * 64] * 700 + [8 * 65]],
+                         ids=["few", "mixed_lengths", "more_than_slots"])
+@pytest.mark.parametrize("small", [0, 1500], ids=["chains_only", "beside_mixed_tiles"])
+def test_short_chains_alone_or_packed(cuda_lib, lens, small):
+    """CBC encryptions of up to 512 blocks, walked one per warp while that ends
+    sooner than 32 to a warp, alone and beside mixed-key tiles (whose kernel
+    overlaps the chains'): every message against the oracle, launched twice."""
+    n = len(lens) + small
+    nbytes = np.array(lens + [8 * (1 + i % 32) for i in range(small)], dtype=np.int64)
+    modes = np.array([4] * len(lens) + [(0, 2, 3)[i % 3] for i in range(small)], dtype=np.uint32)
+    keys = synth.key_triples(n, 37)
+    offs = np.concatenate([[0], np.cumsum(nbytes)])
+    data = synth.random_bytes(n, int(offs[-1]))
+    src = torch.from_numpy(data).cuda()
+    dst = torch.zeros_like(src)
+    ivs = synth.u64s(n, n, synth.STREAM_IV) & np.uint64(0xFFFFFFFF0000FFFF)
+    kt = cuda_lib.KeyTable(keys)
+    ents = [(int(modes[i]), i % 37, int(ivs[i]), src.data_ptr() + int(offs[i]),
+             dst.data_ptr() + int(offs[i]), int(nbytes[i])) for i in range(n)]
+    plan = cuda_lib.Batch(kt, ents)
+    for launch in (plan.launch, plan.launch_graph):
+        dst.zero_()
+        launch()
+        torch.cuda.synchronize()
+        got = dst.cpu().numpy()
+        for i in range(n):
+            k, v, d = keys[i % 37].tobytes(), int(ivs[i]), data[offs[i]:offs[i + 1]]
+            want = (oracle.tdes_ecb(k, d) if modes[i] == 0
+                    else oracle.tdes_ctr(k, v >> 32, v & 0xFFFFFFFF, d) if modes[i] == 2
+                    else oracle.tdes_cbc_decrypt(k, v, d) if modes[i] == 3
+                    else oracle.tdes_cbc_encrypt(k, v, d))
+            assert np.array_equal(got[offs[i]:offs[i + 1]], want), i
