@@ -52,7 +52,7 @@ constexpr uint64_t kSoloChainBlocks = 512;                // longer CBC-enc chai
 // What the choice for shorter chains weighs, in ns: a block of a chain that a
 // warp walks alone (one such chain per SM sub-partition at a time), a block of
 // one of 32 that share a warp, and a tile's share of a sub-partition.
-constexpr uint64_t kSoloBlockNs = 920, kPackedBlockNs = 3400, kTileNs = 12000;
+constexpr uint64_t kSoloBlockNs = 800, kPackedBlockNs = 4000, kTileNs = 12000;
 constexpr uint64_t kSubPartitions = 608;
 constexpr int kPerKeyWords = 2 * TDES_TABLE_WORDS;        // enc + dec bitsliced tables
 constexpr int kPerKeyChunks = 2 * TDES_SUBKEY_WORDS;      // enc + dec scalar groups
@@ -461,9 +461,33 @@ __device__ __forceinline__ void lane_chain(const BatchMsg& m, const SharedTables
     }
 }
 
+__device__ const uint32_t kChainLaneSbox[32][4] = TDES_LANE_SBOX_INIT;
+static_assert(48 * 32 * sizeof(uint2) + TDES_SUBKEY_WORDS <= kWarpSmemBytes,
+              "a chain's tables and key groups fit a warp's slice");
+
+// One chain walked by the calling warp: its tables in the warp's slice, built
+// from the key groups staged behind them.  A real call: inlined in the batch
+// kernel the loop's registers would be allocated with the tiles' planes.
+template <int ROUNDS>
+__device__ __noinline__ void batch_chain_warp(const uint8_t* in, uint8_t* out, uint64_t nblocks,
+                                              uint64_t iv, const uint8_t* __restrict__ kg,
+                                              uint32_t warp, uint32_t lane) {
+    uint8_t* warp_smem = g_dyn + (size_t)warp * kWarpSmemBytes;  // here: known to be shared
+    uint2* tab = reinterpret_cast<uint2*>(warp_smem);
+    uint8_t* keys = warp_smem + 48 * 32 * sizeof(uint2);
+    if (lane < TDES_SUBKEY_WORDS / 16)
+        reinterpret_cast<uint4*>(keys)[lane] = __ldg(reinterpret_cast<const uint4*>(kg) + lane);
+    __syncwarp();
+    const ChainLane c = {kChainLaneSbox[lane][0], kChainLaneSbox[lane][1], kChainLaneSbox[lane][2],
+                         kChainLaneSbox[lane][3]};
+    chain_tables<ROUNDS>(tab, c, keys, lane, 0, 1);
+    __syncwarp();
+    chain_walk<ROUNDS>(in, out, nblocks, iv, c.rot, lane, tab);
+}
+
 // C item: CBC-encryption chains.  The first n_c_solo items (the longest
-// chains) hold one chain each, walked by the whole warp (tdes_block_warp: a
-// ballot per round, so the dependent chain per block is short); the rest hold
+// chains) hold one chain each, walked by the whole warp (chain_walk: a ballot
+// per round, so the dependent chain per block is short); the rest hold
 // up to 32 short chains, one per lane, with the scalar round.
 __device__ __noinline__ void batch_cbc_enc_item(const BatchParams& p, uint32_t item,
                                                 uint32_t warp, uint32_t lane) {
@@ -472,13 +496,10 @@ __device__ __noinline__ void batch_cbc_enc_item(const BatchParams& p, uint32_t i
     if (item < p.n_c_solo) {
         const BatchMsg m = p.msgs[p.c_list[item]];
         const uint8_t* kg = p.keychunks + (uint64_t)m.key * kPerKeyChunks;
-        for (int i = lane; i < TDES_SUBKEY_WORDS / 16; i += 32)
-            reinterpret_cast<uint4*>(warp_smem)[i] = __ldg(reinterpret_cast<const uint4*>(kg) + i);
-        __syncwarp();
         if (p.keystages[m.key] == 1)
-            tdes_cbc_chain_warp<16>(m.in, m.out, m.nblocks, m.iv, warp_smem, lane);
+            batch_chain_warp<16>(m.in, m.out, m.nblocks, m.iv, kg, warp, lane);
         else
-            tdes_cbc_chain_warp<48>(m.in, m.out, m.nblocks, m.iv, warp_smem, lane);
+            batch_chain_warp<48>(m.in, m.out, m.nblocks, m.iv, kg, warp, lane);
         __syncwarp();
         return;
     }

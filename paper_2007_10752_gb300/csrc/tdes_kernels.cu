@@ -593,54 +593,32 @@ cudaError_t launch_cbc_dec(const uint32_t* tab_dec, const uint8_t* chunks, int s
 }
 
 // --------------------------------------------------------------- CBC encrypt
-// C_i = E(P_i XOR C_{i-1}): serial.  One warp walks the chain cooperatively
-// (tdes_block_warp: each lane one bit of the round function, a ballot per
-// round); the next plaintext block is loaded one block ahead.
+// C_i = E(P_i XOR C_{i-1}): serial.  The CTA's warps fold the key into the
+// tables of the chain (tdes_scalar.cuh), then one warp walks it.
 __device__ const uint32_t kLaneSbox[32][4] = TDES_LANE_SBOX_INIT;
-__device__ const uint32_t kLaneIP[32][2] = TDES_LANE_IP_INIT;
-__device__ const uint32_t kLaneFP[32][2] = TDES_LANE_FP_INIT;
-
-__device__ __forceinline__ LaneConsts lane_consts(uint32_t lane) {
-    LaneConsts c;
-    c.mlo = kLaneSbox[lane][0];
-    c.mhi = kLaneSbox[lane][1];
-    c.rot = kLaneSbox[lane][2];
-    c.keypos = kLaneSbox[lane][3];
-    c.ip_hi = kLaneIP[lane][0];
-    c.ip_lo = kLaneIP[lane][1];
-    c.fp_hi = kLaneFP[lane][0];
-    c.fp_lo = kLaneFP[lane][1];
-    return c;
-}
+constexpr int kChainThreads = 512;  // 16 warps: three rounds' tables each
 
 template <int ROUNDS>
-__global__ void tdes_cbc_enc_kernel(const uint8_t* __restrict__ chunks_g, uint64_t iv,
-                                    const uint8_t* in, uint8_t* out, uint64_t nblocks) {
-    __shared__ __align__(16) uint8_t keys[TDES_SUBKEY_WORDS];
+__global__ void __launch_bounds__(kChainThreads)
+tdes_cbc_enc_kernel(const uint8_t* __restrict__ chunks_g, uint64_t iv, const uint8_t* in,
+                    uint8_t* out, uint64_t nblocks) {
+    __shared__ uint2 tab[32 * ROUNDS];
     const uint32_t lane = threadIdx.x & 31u;
-    for (int i = threadIdx.x; i < TDES_SUBKEY_WORDS; i += blockDim.x) keys[i] = chunks_g[i];
+    const ChainLane c = {kLaneSbox[lane][0], kLaneSbox[lane][1], kLaneSbox[lane][2],
+                         kLaneSbox[lane][3]};
+    chain_tables<ROUNDS>(tab, c, chunks_g, lane, threadIdx.x >> 5, blockDim.x >> 5);
     __syncthreads();
     if (threadIdx.x >= 32) return;
-    const LaneConsts c = lane_consts(lane);
-    const uint64_t* p = reinterpret_cast<const uint64_t*>(in);
-    uint64_t* q = reinterpret_cast<uint64_t*>(out);
-    uint64_t prev = iv;
-    uint64_t next = p[0];
-    for (uint64_t i = 0; i < nblocks; ++i) {
-        const uint64_t x = bswap64(next) ^ prev;
-        if (i + 1 < nblocks) next = p[i + 1];
-        prev = tdes_block_warp<ROUNDS>(x, c, keys);
-        if (lane == 0) q[i] = bswap64(prev);
-    }
+    chain_walk<ROUNDS>(in, out, nblocks, iv, c.rot, lane, tab);
 }
 
 cudaError_t launch_cbc_enc(const uint8_t* chunk_enc, int stages, uint64_t iv, const void* in,
                            void* out, uint64_t nblocks, cudaStream_t s) {
     if (stages == 1)
-        tdes_cbc_enc_kernel<16><<<1, 32, 0, s>>>(chunk_enc, iv, static_cast<const uint8_t*>(in),
+        tdes_cbc_enc_kernel<16><<<1, kChainThreads, 0, s>>>(chunk_enc, iv, static_cast<const uint8_t*>(in),
                                                  static_cast<uint8_t*>(out), nblocks);
     else
-        tdes_cbc_enc_kernel<48><<<1, 32, 0, s>>>(chunk_enc, iv, static_cast<const uint8_t*>(in),
+        tdes_cbc_enc_kernel<48><<<1, kChainThreads, 0, s>>>(chunk_enc, iv, static_cast<const uint8_t*>(in),
                                                  static_cast<uint8_t*>(out), nblocks);
     return cudaGetLastError();
 }

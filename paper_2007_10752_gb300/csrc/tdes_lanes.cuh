@@ -32,29 +32,6 @@ struct LaneKeys {  // 48 rounds x (ke, ko), by value
     uint32_t w[TDES_SUBKEY_WORDS / 4];
 };
 
-// IP and FP as swaps of bit groups between the halves: IP is a transpose of
-// the block's 8x8 bit matrix followed by a row reordering, and each of its
-// five steps exchanges one index bit.
-__device__ __forceinline__ void bit_swap(uint32_t& a, uint32_t& b, int n, uint32_t m) {
-    const uint32_t t = ((a >> n) ^ b) & m;
-    b ^= t;
-    a ^= t << n;
-}
-__device__ __forceinline__ void swap_ip(uint32_t& l, uint32_t& r) {
-    bit_swap(l, r, 4, 0x0F0F0F0Fu);
-    bit_swap(l, r, 16, 0x0000FFFFu);
-    bit_swap(r, l, 2, 0x33333333u);
-    bit_swap(r, l, 8, 0x00FF00FFu);
-    bit_swap(l, r, 1, 0x55555555u);
-}
-__device__ __forceinline__ void swap_fp(uint32_t& l, uint32_t& r) {
-    bit_swap(l, r, 1, 0x55555555u);
-    bit_swap(r, l, 8, 0x00FF00FFu);
-    bit_swap(r, l, 2, 0x33333333u);
-    bit_swap(l, r, 16, 0x0000FFFFu);
-    bit_swap(l, r, 4, 0x0F0F0F0Fu);
-}
-
 // Fills the tables: sp is the 8 x 64 words of TDES_SP_INIT.  Row i / 8 of the
 // 16-byte stores is a (q, x, h); eight stores fill its 32 lanes' copies.
 __device__ __forceinline__ void lane_tables(uint8_t* __restrict__ tab,

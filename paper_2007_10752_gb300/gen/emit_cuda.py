@@ -417,13 +417,6 @@ def emit(path: str = OUT) -> str:
         pos = SCALAR_GROUP_ORDER.index(g)
         L.append(f"  {{0x{mask & 0xFFFFFFFF:08x}u, 0x{mask >> 32:08x}u, {rot}u, {pos}u}}, \\")
     L.append("}")
-    L.append("// Per lane l: 0-based source bit of output bits 32 - l and 64 - l of IP and FP.")
-    for name, perm in (("IP", T.IP), ("FP", T.FP)):
-        L.append(f"#define TDES_LANE_{name}_INIT {{ \\")
-        L.append("  " + ", ".join("{%du, %du}" % (perm[32 - l - 1] - 1, perm[64 - l - 1] - 1)
-                               for l in range(32)) + " \\")
-        L.append("}")
-    L.append("")
     L.append("// Initial / final permutation by nibbles: entry [n][v] is the output word")
     L.append("// contribution of value v in input nibble n (input bits 4n+1..4n+4).")
     for name, perm in (("IPN", T.IP), ("FPN", T.FP)):
