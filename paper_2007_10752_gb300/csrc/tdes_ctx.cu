@@ -339,18 +339,18 @@ int tdes_batch_poll(tdes_ctx_t* c, uint64_t ticket, int* per_desc_status) {
 int tdes_batch_wait(tdes_ctx_t* c, uint64_t ticket, uint64_t timeout_ns) {
     const int64_t start = now_ns();
     const int64_t until = start + (int64_t)std::min<uint64_t>(timeout_ns, INT64_MAX / 4);
-    int64_t nap_ns = 2000;
     for (;;) {
         const int r = tdes_batch_poll(c, ticket, nullptr);
         if (r != 1) return r;
         const int64_t now = now_ns();
         if (now >= until)
             return cfail(TDES_ETIMEDOUT, "ticket %llu still pending", (unsigned long long)ticket);
-        // short naps first (a batch of small messages completes in tens of
-        // microseconds), then longer ones: the thread does not spin
+        // Naps of an eighth of the time waited so far, 2 us to 1 ms: the thread
+        // does not spin, and learns of a completion within an eighth of its time
+        // (doubling naps saw a batch of 0.64 ms only at 0.95 ms).
+        const int64_t nap_ns = std::max<int64_t>(2000, std::min<int64_t>((now - start) / 8, 1000000));
         std::this_thread::sleep_for(
             std::chrono::nanoseconds(std::min<int64_t>(nap_ns, until - now)));
-        nap_ns = std::min<int64_t>(nap_ns * 2, 1000000);
     }
 }
 

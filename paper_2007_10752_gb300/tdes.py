@@ -10,6 +10,8 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
+from itertools import chain
 
 import numpy as np
 
@@ -258,10 +260,29 @@ def _nbytes(t) -> int:
     return t.numel() * t.element_size()
 
 
+_raw_stream = None  # (current device, its current stream's address), once CUDA is up
+
+
+def _current_stream() -> int:
+    """Address of torch's current stream on the current device.  torch's own
+    accessor builds a Stream object (with the import 4.7 us a call, half of a small call's
+    host time); the address alone takes 0.3 us."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        s = torch.cuda.current_stream().cuda_stream  # initialises CUDA
+        device = getattr(torch._C, "_cuda_getDevice", None)
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        _raw_stream = ((device, raw) if device and raw else
+                       (lambda: None, lambda _: torch.cuda.current_stream().cuda_stream))
+        return s
+    device, raw = _raw_stream
+    return raw(device())
+
+
 def _stream(stream) -> int:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -426,10 +447,21 @@ class KeyTable:
 def make_descs(entries):
     """entries: iterable of (mode, key_index, iv_or_ctr, in_ptr, out_ptr, nbytes)."""
     entries = list(entries)
-    arr = (Desc * max(1, len(entries)))()
-    for i, (mode, key, iv, ip, op, n) in enumerate(entries):
-        arr[i] = Desc(mode, key, iv & (2**64 - 1), _ptr(ip), _ptr(op), n)
-    return arr, len(entries)
+    n = len(entries)
+    arr = (Desc * max(1, n))()
+    flat = (list(chain.from_iterable(entries))
+            if set(map(type, entries)) <= {tuple, list} and set(map(len, entries)) <= {6} else ())
+    if len(flat) == 6 * n and set(map(type, flat)) <= {int}:
+        # plain numbers: one pack call for all (1024 entries: 0.22 against 0.61 ms);
+        # a number out of its field's range takes the general path below
+        try:
+            struct.pack_into("<" + "IIQQQQ" * n, arr, 0, *flat)
+            return arr, n
+        except struct.error:
+            pass
+    for i, (mode, key, iv, ip, op, nb) in enumerate(entries):
+        arr[i] = Desc(mode, key, iv & (2**64 - 1), _ptr(ip), _ptr(op), nb)
+    return arr, n
 
 
 DESC_DTYPE = np.dtype([("mode", "<u4"), ("key_index", "<u4"), ("iv_or_ctr", "<u8"),
@@ -714,7 +746,7 @@ class Server:
         t = ctypes.c_uint64()
         _check(load().tdes_server_submit_group(self.handle, ctypes.addressof(arr), n,
                                                ctypes.byref(t)))
-        self._hold(t.value, n, [b for e in entries for b in (e[3], e[4])])
+        self._hold(t.value, n, [b for e in entries for b in e[3:5] if not isinstance(b, int)])
         return t.value, n
 
     def poll_group(self, group) -> tuple:
