@@ -265,8 +265,8 @@ _raw_stream = None  # (current device, its current stream's address), once CUDA 
 
 def _current_stream() -> int:
     """Address of torch's current stream on the current device.  torch's own
-    accessor builds a Stream object (with the import 4.7 us a call, half of a small call's
-    host time); the address alone takes 0.3 us."""
+    accessor builds a Stream object (with the import 4.7 us a call, half of a
+    small call's host time); the address alone takes 0.3 us."""
     global _raw_stream
     if _raw_stream is None:
         import torch
