@@ -60,8 +60,6 @@ constexpr int kWarpSmemBytes = TDES_TABLE_WORDS * 4;      // one table per warp 
 static_assert(32 * TDES_SUBKEY_WORDS <= kWarpSmemBytes, "scalar groups must fit a warp slice");
 
 __device__ const uint32_t kBatchSP[8][64] = TDES_SP_INIT;
-__device__ const uint64_t kBatchIPN[16][16] = TDES_IPN_INIT;
-__device__ const uint64_t kBatchFPN[16][16] = TDES_FPN_INIT;
 __device__ const uint8_t kBatchRecipe[2][TDES_TABLE_WORDS][3] = TDES_RECIPE_INIT;
 __device__ const uint8_t kBatchRecipe1[2][TDES1_TABLE_WORDS][3] = TDES1_RECIPE_INIT;
 __device__ const uint8_t kBatchSubkeyBits[2][48][48] = TDES_SUBKEY_INIT;
@@ -130,8 +128,6 @@ __global__ void tdes_keytable_pack_kernel(const uint8_t* __restrict__ keys, uint
 
 struct SharedTables {
     uint32_t sp[8 * 64];
-    uint64_t ipn[16 * 16];
-    uint64_t fpn[16 * 16];
 };
 
 // Shared memory of the batch kernel, at namespace scope so that the scalar
@@ -323,8 +319,8 @@ __device__ __noinline__ void batch_scalar_item(const BatchParams& p, uint2 item,
     if (msg != 0xFFFFFFFFu) {
         const uint32_t* ks = reinterpret_cast<const uint32_t*>(warp_smem + TDES_SUBKEY_WORDS * lane);
         uint64_t y = p.keystages[m.key] == 1
-                         ? tdes_block_scalar_nib<16>(x, st.sp, ks, st.ipn, st.fpn)
-                         : tdes_block_scalar_nib<48>(x, st.sp, ks, st.ipn, st.fpn);
+                         ? tdes_block_scalar_swap<16>(x, st.sp, ks)
+                         : tdes_block_scalar_swap<48>(x, st.sp, ks);
         if (m.mode == TDES_MODE_CTR || m.mode == TDES_MODE_CBC_DECRYPT) y ^= prev;
         store_be(m.out, blk, y);
     }
@@ -456,7 +452,7 @@ __device__ __forceinline__ void lane_chain(const BatchMsg& m, const SharedTables
     for (uint64_t i = 0; i < m.nblocks; ++i) {
         const uint64_t x = next ^ prev;
         if (i + 1 < m.nblocks) next = load_be(m.in, i + 1);
-        prev = tdes_block_scalar_nib<ROUNDS>(x, st.sp, keys, st.ipn, st.fpn);
+        prev = tdes_block_scalar_swap<ROUNDS>(x, st.sp, keys);
         store_be(m.out, i, prev);
     }
 }
@@ -533,10 +529,6 @@ template <bool SOLO_SLOTS, bool COMPACT>
 __global__ void __launch_bounds__(256, 2) tdes_batch_kernel(BatchParams p) {
     if (p.n_m_tiles == 0) stamp_start(p);  // else the mixed-key kernel ran first
     for (int i = threadIdx.x; i < 8 * 64; i += blockDim.x) g_st.sp[i] = (&kBatchSP[0][0])[i];
-    for (int i = threadIdx.x; i < 16 * 16; i += blockDim.x) {
-        g_st.ipn[i] = (&kBatchIPN[0][0])[i];
-        g_st.fpn[i] = (&kBatchFPN[0][0])[i];
-    }
     __syncthreads();
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     uint32_t* wtab = reinterpret_cast<uint32_t*>(g_dyn + (size_t)warp * kWarpSmemBytes);

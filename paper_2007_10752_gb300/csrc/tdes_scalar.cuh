@@ -77,7 +77,8 @@ TDES_HD uint64_t permute64_nib(uint64_t v, const uint64_t* __restrict__ tab) {
 }
 
 // The same EDE3 block as tdes_block_scalar with the permutations by nibble
-// tables (ipn/fpn: 16 x 16 words each) instead of bit loops.  The 16 rounds
+// tables (ipn/fpn: 16 x 16 words each) instead of bit loops; the host check's
+// form (the kernels take tdes_block_scalar_swap).  The 16 rounds
 // of a DES pass are unrolled by two so that the halves alternate in place,
 // and each round's key words are loaded one round ahead, off the chain of
 // dependent operations that sets the latency of a block.
@@ -128,6 +129,32 @@ TDES_HD void swap_fp(uint32_t& l, uint32_t& r) {
     bit_swap(r, l, 2, 0x33333333u);
     bit_swap(l, r, 16, 0x0000FFFFu);
     bit_swap(l, r, 4, 0x0F0F0F0Fu);
+}
+
+// tdes_block_scalar_nib with the permutations as bit swaps: no tables to stage
+// and no lookups for them.
+template <int ROUNDS = 48>
+TDES_HD uint64_t tdes_block_scalar_swap(uint64_t v, const uint32_t* __restrict__ sp,
+                                        const uint32_t* __restrict__ keys) {
+    uint32_t L = (uint32_t)(v >> 32), R = (uint32_t)v;
+    swap_ip(L, R);
+    uint32_t ke = keys[0], ko = keys[1];
+#pragma unroll
+    for (int r = 0; r < ROUNDS; r += 2) {
+        const uint32_t ke1 = keys[2 * r + 2], ko1 = keys[2 * r + 3];
+        L ^= tdes_f_scalar(R, ke, ko, sp);
+        const int rn = r + 2 < ROUNDS ? r + 2 : r;  // the last prefetch rereads the last pair
+        ke = keys[2 * rn];
+        ko = keys[2 * rn + 1];
+        R ^= tdes_f_scalar(L, ke1, ko1, sp);
+        if ((r & 15) == 14) {  // end of a DES pass: R16 || L16 continues as the next L0 || R0
+            const uint32_t u = L;
+            L = R;
+            R = u;
+        }
+    }
+    swap_fp(L, R);
+    return ((uint64_t)L << 32) | R;
 }
 
 TDES_HD uint64_t bswap64(uint64_t x) {

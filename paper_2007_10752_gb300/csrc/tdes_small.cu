@@ -6,11 +6,12 @@
 // A bitsliced tile is 1024 blocks and costs each lane about 12 k logic
 // operations (48 rounds over 64 bit-planes), so a call of a few tiles takes
 // one tile's latency however few blocks it holds.  Here each thread runs its
-// own block through the scalar round (tdes_block_scalar_nib: the expansion
-// windows as two rotates, eight S-box/permutation table lookups, nibble
-// tables for IP and FP), a chain of 48 dependent rounds (16 for single DES).
-// The tables and the call's round-key words are staged in shared memory once
-// per CTA.
+// own block through the scalar round (tdes_block_scalar_swap: the expansion
+// windows as two rotates, eight S-box/permutation table lookups, IP and FP as
+// bit swaps), a chain of 48 dependent rounds (16 for single DES).
+// The table and the call's round-key words are staged in shared memory once
+// per CTA: 2.4 KB, where nibble tables for IP and FP made it 6.4 KB (a call of
+// 64 blocks 4.04 -> 3.52 us, of 24576 6.14 -> 5.48 us, device time).
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -23,14 +24,10 @@
 
 namespace tdes {
 
-__device__ const uint32_t kSmallSP[8][64] = TDES_SP_INIT;
-__device__ const uint64_t kSmallIPN[16][16] = TDES_IPN_INIT;
-__device__ const uint64_t kSmallFPN[16][16] = TDES_FPN_INIT;
+__device__ const __align__(16) uint32_t kSmallSP[8][64] = TDES_SP_INIT;
 
 struct SmallTables {
     uint32_t sp[8 * 64];
-    uint64_t ipn[16 * 16];
-    uint64_t fpn[16 * 16];
     uint32_t keys[TDES_SUBKEY_WORDS / 4];
 };
 
@@ -49,11 +46,8 @@ __global__ void __launch_bounds__(1024)
 tdes_small_kernel(const uint8_t* __restrict__ chunks, int mode, uint64_t iv, const uint8_t* in,
                   uint8_t* out, uint64_t nblocks) {
     __shared__ __align__(16) SmallTables st;
-    for (int i = threadIdx.x; i < 8 * 64; i += blockDim.x) st.sp[i] = (&kSmallSP[0][0])[i];
-    for (int i = threadIdx.x; i < 16 * 16; i += blockDim.x) {
-        st.ipn[i] = (&kSmallIPN[0][0])[i];
-        st.fpn[i] = (&kSmallFPN[0][0])[i];
-    }
+    for (int i = threadIdx.x; i < 8 * 64 / 4; i += blockDim.x)
+        reinterpret_cast<uint4*>(st.sp)[i] = __ldg(reinterpret_cast<const uint4*>(&kSmallSP[0][0]) + i);
     for (int i = threadIdx.x; i < TDES_SUBKEY_WORDS / 4; i += blockDim.x)
         st.keys[i] = __ldg(reinterpret_cast<const uint32_t*>(chunks) + i);
     const uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -69,7 +63,7 @@ tdes_small_kernel(const uint8_t* __restrict__ chunks, int mode, uint64_t iv, con
     }
     __syncthreads();  // tables staged; every read of this CTA precedes its writes
     if (b < nblocks) {
-        uint64_t y = tdes_block_scalar_nib<ROUNDS>(x, st.sp, st.keys, st.ipn, st.fpn);
+        uint64_t y = tdes_block_scalar_swap<ROUNDS>(x, st.sp, st.keys);
         if (mode != kSmallEcb) y ^= prev;
         reinterpret_cast<uint64_t*>(out)[b] = bswap64(y);
     }
@@ -105,8 +99,8 @@ tdes_lanes_kernel(const __grid_constant__ LaneKeys keys, int mode, uint64_t iv, 
 
 // Whether a call takes tdes_lanes_kernel.  Below kLanesMinBlocks the few warps
 // an SM has do not fill its shared memory's cycles and writing 64 KB of tables
-// costs more than the conflicts (16384 blocks: 6.8 us against 4.8 us of
-// tdes_small_kernel; 24576: 6.2 against 6.1; 32768: 5.1 against 6.2).  CBC
+// costs more than the conflicts (16384 blocks: 6.8 us against 4.3 us of
+// tdes_small_kernel; 24576: 6.2 against 5.5; 32768: 5.1 against over 6).  CBC
 // decryption only out of place: its CTAs write while others still read.
 static bool use_lanes(int mode, const void* in, const void* out, uint64_t nblocks) {
     return nblocks > kLanesMinBlocks && nblocks <= (1ull << 30) &&
