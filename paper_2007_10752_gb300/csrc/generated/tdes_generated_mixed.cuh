@@ -61,32 +61,31 @@ TDES_HD void tdes_round_mixed(uint32_t (&T)[32], const uint32_t (&S)[32],
     const uint32_t x4 = S[7];
     const uint32_t x5 = S[8];
     const uint4 kc = *reinterpret_cast<const uint4*>(k + 8);
-    const uint32_t s1_0 = lop3<0xb1>(x4, x1, x0);
-    const uint32_t s1_1 = lop3<0x43>(x5, s1_0, x1);
-    const uint32_t s1_2 = lop3<0xbd>(x1, x5, x0);
-    const uint32_t s1_3 = lop3<0x84>(s1_2, x4, x0);
-    const uint32_t s1_4 = lop3<0x67>(s1_1, s1_0, x0);
-    const uint32_t s1_5 = lop3<0x16>(s1_4, x4, x1);
-    const uint32_t s1_6 = lop3<0x6f>(s1_4, s1_5, x5);
-    const uint32_t s1_7 = lop3<0xa6>(s1_5, x3, x2);
-    const uint32_t s1_8 = lop3<0x67>(s1_2, s1_7, s1_3);
-    const uint32_t s1_9 = lop3<0x95>(s1_6, s1_8, x3);
-    T[17] = lop3<0x96>(T[17], s1_9, kc.w);
-    const uint32_t s1_10 = lop3<0xb6>(s1_9, x5, x0);
-    const uint32_t s1_11 = lop3<0x58>(s1_5, s1_3, x2);
-    const uint32_t s1_12 = lop3<0x9a>(s1_10, s1_4, x4);
-    const uint32_t s1_13 = lop3<0x69>(s1_12, s1_1, s1_7);
-    T[12] = lop3<0x96>(T[12], s1_13, kc.x);
-    const uint32_t s1_14 = lop3<0x53>(s1_10, s1_13, x0);
-    const uint32_t s1_15 = lop3<0xe9>(s1_14, s1_13, s1_2);
-    const uint32_t s1_16 = lop3<0xe5>(s1_14, s1_13, x5);
-    const uint32_t s1_17 = lop3<0x0c>(s1_13, s1_2, s1_0);
-    const uint32_t s1_18 = lop3<0x6c>(s1_16, s1_17, x4);
-    const uint32_t s1_19 = lop3<0x69>(s1_18, s1_9, x1);
-    T[27] = lop3<0x69>(T[27], s1_19, kc.y);
-    const uint32_t s1_20 = lop3<0x8d>(s1_15, s1_11, s1_9);
-    const uint32_t s1_21 = lop3<0x49>(s1_12, s1_16, s1_20);
-    T[1] = lop3<0x96>(T[1], s1_21, kc.z);
+    const uint32_t s1_0 = lop3<0x38>(x5, x2, x1);
+    const uint32_t s1_1 = lop3<0x78>(x4, x3, x1);
+    const uint32_t s1_2 = lop3<0x96>(s1_1, s1_0, x3);
+    const uint32_t s1_3 = lop3<0x84>(x3, s1_1, x5);
+    const uint32_t s1_4 = lop3<0x05>(s1_3, x3, x1);
+    const uint32_t s1_5 = lop3<0x4a>(x5, s1_4, x0);
+    const uint32_t s1_6 = lop3<0xad>(s1_5, s1_4, s1_1);
+    const uint32_t s1_7 = lop3<0xd0>(s1_5, x5, x1);
+    const uint32_t s1_8 = lop3<0xc5>(s1_7, x2, x4);
+    const uint32_t s1_9 = lop3<0x46>(s1_8, s1_0, x0);
+    const uint32_t s1_10 = lop3<0x2d>(s1_6, s1_9, x2);
+    T[12] = lop3<0x69>(T[12], s1_10, kc.x);
+    const uint32_t s1_11 = lop3<0xe9>(s1_10, s1_5, x0);
+    const uint32_t s1_12 = lop3<0x31>(s1_10, s1_4, s1_8);
+    const uint32_t s1_13 = lop3<0x04>(s1_12, s1_11, x4);
+    const uint32_t s1_14 = lop3<0x96>(s1_5, s1_13, s1_2);
+    T[17] = lop3<0x96>(T[17], s1_14, kc.w);
+    const uint32_t s1_15 = lop3<0x67>(s1_12, s1_3, s1_0);
+    const uint32_t s1_16 = lop3<0xac>(s1_15, s1_6, s1_2);
+    const uint32_t s1_17 = lop3<0x69>(s1_16, x1, x0);
+    T[27] = lop3<0x96>(T[27], s1_17, kc.y);
+    const uint32_t s1_18 = lop3<0x92>(s1_16, x5, x1);
+    const uint32_t s1_19 = lop3<0xf9>(s1_18, s1_14, s1_5);
+    const uint32_t s1_20 = lop3<0x96>(s1_19, s1_11, s1_8);
+    T[1] = lop3<0x69>(T[1], s1_20, kc.z);
     }
     {  // S-box 3
     const uint4 kd = *reinterpret_cast<const uint4*>(k + 20);
@@ -163,35 +162,32 @@ TDES_HD void tdes_round_mixed(uint32_t (&T)[32], const uint32_t (&S)[32],
     const uint32_t x4 = S[19];
     const uint32_t x5 = S[20];
     const uint4 kc = *reinterpret_cast<const uint4*>(k + 32);
-    const uint32_t s4_0 = lop3<0x25>(x5, x3, x0);
-    const uint32_t s4_1 = lop3<0x68>(s4_0, x2, x0);
-    const uint32_t s4_2 = lop3<0x82>(s4_1, x4, x2);
-    const uint32_t s4_3 = lop3<0x4a>(s4_2, x0, x3);
-    const uint32_t s4_4 = lop3<0x49>(s4_2, x3, x0);
-    const uint32_t s4_5 = lop3<0x9a>(x4, s4_1, s4_4);
-    const uint32_t s4_6 = lop3<0xb9>(s4_4, x2, s4_0);
-    const uint32_t s4_7 = lop3<0x75>(s4_6, x3, x1);
-    const uint32_t s4_8 = lop3<0x34>(s4_5, s4_3, x0);
-    const uint32_t s4_9 = lop3<0xe9>(s4_8, x2, x5);
-    const uint32_t s4_10 = lop3<0x69>(s4_9, s4_3, s4_7);
-    T[13] = lop3<0x96>(T[13], s4_10, kc.y);
-    const uint32_t s4_11 = lop3<0x24>(s4_10, s4_7, x3);
-    const uint32_t s4_12 = lop3<0x7e>(s4_10, s4_5, x5);
-    const uint32_t s4_13 = lop3<0x5a>(s4_9, x5, x3);
-    const uint32_t s4_14 = lop3<0x9d>(s4_13, x4, x0);
-    const uint32_t s4_15 = lop3<0x82>(s4_14, s4_6, s4_7);
-    const uint32_t s4_16 = lop3<0x52>(s4_15, s4_4, x1);
-    T[24] = lop3<0x96>(T[24], s4_16, kc.z);
-    const uint32_t s4_17 = lop3<0x43>(s4_16, s4_15, s4_12);
-    const uint32_t s4_18 = lop3<0x2c>(s4_17, s4_13, s4_7);
-    const uint32_t s4_19 = lop3<0x8c>(s4_12, s4_11, x5);
-    const uint32_t s4_20 = lop3<0x96>(s4_19, s4_18, x1);
-    const uint32_t s4_21 = lop3<0xd2>(s4_20, x4, x1);
-    T[2] = lop3<0x96>(T[2], s4_21, kc.w);
-    const uint32_t s4_22 = lop3<0xb9>(x4, s4_21, s4_10);
-    const uint32_t s4_23 = lop3<0x14>(s4_22, s4_16, s4_8);
-    const uint32_t s4_24 = lop3<0xa6>(s4_23, s4_12, x1);
-    T[7] = lop3<0x69>(T[7], s4_24, kc.x);
+    const uint32_t s4_0 = lop3<0x82>(x4, x2, x0);
+    const uint32_t s4_1 = lop3<0x49>(x5, x3, x2);
+    const uint32_t s4_2 = lop3<0xc2>(x4, s4_0, s4_1);
+    const uint32_t s4_3 = lop3<0x29>(x2, s4_2, x3);
+    const uint32_t s4_4 = lop3<0xc9>(s4_2, x5, x0);
+    const uint32_t s4_5 = lop3<0x61>(s4_4, x4, x3);
+    const uint32_t s4_6 = lop3<0x16>(s4_2, x5, x2);
+    const uint32_t s4_7 = lop3<0x32>(s4_6, s4_3, x4);
+    const uint32_t s4_8 = lop3<0x9e>(s4_4, s4_3, s4_1);
+    const uint32_t s4_9 = lop3<0x8a>(s4_8, x3, x1);
+    const uint32_t s4_10 = lop3<0xa8>(s4_8, s4_0, x4);
+    const uint32_t s4_11 = lop3<0xec>(s4_10, s4_5, s4_1);
+    const uint32_t s4_12 = lop3<0xd2>(s4_11, s4_7, x1);
+    T[2] = lop3<0x69>(T[2], s4_12, kc.w);
+    const uint32_t s4_13 = lop3<0x64>(s4_9, s4_11, s4_7);
+    const uint32_t s4_14 = lop3<0xb6>(s4_13, x4, x0);
+    const uint32_t s4_15 = lop3<0x7c>(s4_13, s4_8, s4_3);
+    const uint32_t s4_16 = lop3<0x95>(s4_9, s4_15, s4_6);
+    const uint32_t s4_17 = lop3<0xa5>(s4_9, s4_2, s4_1);
+    const uint32_t s4_18 = lop3<0x96>(s4_17, s4_10, x0);
+    T[13] = lop3<0x96>(T[13], s4_18, kc.y);
+    const uint32_t s4_19 = lop3<0x96>(s4_16, s4_14, x1);
+    T[7] = lop3<0x96>(T[7], s4_19, kc.x);
+    const uint32_t s4_20 = lop3<0x69>(s4_19, s4_13, s4_18);
+    const uint32_t s4_21 = lop3<0xc6>(s4_14, s4_20, s4_12);
+    T[24] = lop3<0x69>(T[24], s4_21, kc.z);
     }
     {  // S-box 6
     const uint4 kd = *reinterpret_cast<const uint4*>(k + 44);
@@ -238,33 +234,32 @@ TDES_HD void tdes_round_mixed(uint32_t (&T)[32], const uint32_t (&S)[32],
     const uint32_t x4 = S[27];
     const uint32_t x5 = S[28];
     const uint4 kc = *reinterpret_cast<const uint4*>(k + 48);
-    const uint32_t s6_0 = lop3<0xe7>(x2, x5, x0);
-    const uint32_t s6_1 = lop3<0xa4>(x3, x1, x0);
-    const uint32_t s6_2 = lop3<0x6b>(s6_0, s6_1, x2);
-    const uint32_t s6_3 = lop3<0x96>(s6_2, x5, x1);
-    const uint32_t s6_4 = lop3<0x9f>(x1, s6_3, s6_0);
-    const uint32_t s6_5 = lop3<0x12>(x3, s6_0, x0);
-    const uint32_t s6_6 = lop3<0x47>(x3, s6_3, x2);
-    const uint32_t s6_7 = lop3<0x18>(s6_5, s6_6, x0);
-    const uint32_t s6_8 = lop3<0x39>(s6_7, s6_3, x4);
-    T[31] = lop3<0x69>(T[31], s6_8, kc.x);
-    const uint32_t s6_9 = lop3<0x6c>(s6_8, x2, x1);
-    const uint32_t s6_10 = lop3<0x9a>(s6_4, s6_7, x4);
-    const uint32_t s6_11 = lop3<0xdc>(s6_10, x5, x4);
-    const uint32_t s6_12 = lop3<0xb6>(x1, s6_11, s6_0);
-    const uint32_t s6_13 = lop3<0x49>(s6_9, x0, x1);
-    const uint32_t s6_14 = lop3<0x52>(s6_13, s6_10, s6_2);
-    const uint32_t s6_15 = lop3<0xa3>(s6_11, s6_9, x3);
-    const uint32_t s6_16 = lop3<0xe2>(s6_14, s6_15, s6_12);
-    T[21] = lop3<0x96>(T[21], s6_16, kc.z);
-    const uint32_t s6_17 = lop3<0x62>(s6_8, s6_0, x0);
-    const uint32_t s6_18 = lop3<0xe9>(s6_17, s6_11, s6_3);
-    const uint32_t s6_19 = lop3<0x6c>(s6_18, s6_10, x3);
-    T[11] = lop3<0x96>(T[11], s6_19, kc.y);
-    const uint32_t s6_20 = lop3<0xf4>(s6_19, x2, x1);
-    const uint32_t s6_21 = lop3<0x9b>(s6_20, x4, x3);
-    const uint32_t s6_22 = lop3<0x96>(x5, s6_21, s6_13);
-    T[6] = lop3<0x96>(T[6], s6_22, kc.w);
+    const uint32_t s6_0 = lop3<0x69>(x5, x2, x0);
+    const uint32_t s6_1 = lop3<0x93>(x5, x3, x1);
+    const uint32_t s6_2 = lop3<0x5e>(s6_1, x4, x1);
+    const uint32_t s6_3 = lop3<0x81>(s6_1, x3, x0);
+    const uint32_t s6_4 = lop3<0x26>(s6_3, s6_2, x2);
+    const uint32_t s6_5 = lop3<0x52>(x4, s6_4, x3);
+    const uint32_t s6_6 = lop3<0xe1>(s6_5, s6_4, x1);
+    const uint32_t s6_7 = lop3<0xea>(s6_6, x5, x0);
+    const uint32_t s6_8 = lop3<0x69>(s6_7, s6_4, x4);
+    const uint32_t s6_9 = lop3<0x69>(s6_6, x1, x5);
+    const uint32_t s6_10 = lop3<0x36>(s6_6, s6_3, x3);
+    const uint32_t s6_11 = lop3<0x69>(s6_10, s6_9, x2);
+    const uint32_t s6_12 = lop3<0xb8>(s6_0, s6_11, s6_1);
+    const uint32_t s6_13 = lop3<0x69>(s6_12, x1, x4);
+    T[11] = lop3<0x69>(T[11], s6_13, kc.y);
+    const uint32_t s6_14 = lop3<0x0d>(s6_13, s6_6, x5);
+    const uint32_t s6_15 = lop3<0x02>(s6_13, s6_8, x5);
+    const uint32_t s6_16 = lop3<0x39>(s6_15, s6_9, x0);
+    T[6] = lop3<0x96>(T[6], s6_16, kc.w);
+    const uint32_t s6_17 = lop3<0x7d>(s6_14, s6_3, x0);
+    const uint32_t s6_18 = lop3<0xca>(s6_17, s6_8, s6_11);
+    T[21] = lop3<0x96>(T[21], s6_18, kc.z);
+    const uint32_t s6_19 = lop3<0xe1>(s6_13, s6_11, s6_3);
+    const uint32_t s6_20 = lop3<0xf8>(s6_17, x4, x2);
+    const uint32_t s6_21 = lop3<0x67>(s6_1, s6_20, s6_19);
+    T[31] = lop3<0x96>(T[31], s6_21, kc.x);
     }
     {  // S-box 8
     const uint4 kd = *reinterpret_cast<const uint4*>(k + 60);
@@ -275,30 +270,29 @@ TDES_HD void tdes_round_mixed(uint32_t (&T)[32], const uint32_t (&S)[32],
     const uint32_t x4 = S[31];
     const uint32_t x5 = S[0];
     const uint4 kc = *reinterpret_cast<const uint4*>(k + 56);
-    const uint32_t s7_0 = lop3<0xc5>(x5, x3, x0);
-    const uint32_t s7_1 = lop3<0xc6>(s7_0, x4, x1);
-    const uint32_t s7_2 = lop3<0x8b>(x2, s7_0, x1);
-    const uint32_t s7_3 = lop3<0x96>(x4, x3, x2);
-    const uint32_t s7_4 = lop3<0xa9>(s7_1, s7_3, x3);
-    const uint32_t s7_5 = lop3<0x69>(s7_4, x1, x0);
-    const uint32_t s7_6 = lop3<0xe8>(s7_5, s7_4, s7_1);
-    const uint32_t s7_7 = lop3<0x53>(s7_6, s7_4, x1);
-    const uint32_t s7_8 = lop3<0x69>(s7_7, s7_5, s7_3);
-    const uint32_t s7_9 = lop3<0xd6>(s7_8, x5, x4);
-    const uint32_t s7_10 = lop3<0xc6>(s7_9, s7_5, x0);
-    T[14] = lop3<0x96>(T[14], s7_10, kc.z);
-    const uint32_t s7_11 = lop3<0x96>(s7_10, s7_7, x2);
-    const uint32_t s7_12 = lop3<0x53>(s7_7, s7_2, x0);
-    const uint32_t s7_13 = lop3<0x28>(x4, s7_12, x3);
-    const uint32_t s7_14 = lop3<0xf2>(s7_13, s7_11, s7_3);
-    const uint32_t s7_15 = lop3<0x47>(s7_14, s7_10, s7_2);
-    const uint32_t s7_16 = lop3<0x39>(s7_15, s7_8, x5);
-    T[20] = lop3<0x69>(T[20], s7_16, kc.w);
-    const uint32_t s7_17 = lop3<0x96>(s7_14, x1, x5);
-    T[26] = lop3<0x69>(T[26], s7_17, kc.y);
-    const uint32_t s7_18 = lop3<0xd2>(s7_15, s7_6, x0);
-    const uint32_t s7_19 = lop3<0xa6>(x5, s7_18, s7_8);
-    T[4] = lop3<0x69>(T[4], s7_19, kc.x);
+    const uint32_t s7_0 = lop3<0x91>(x1, x4, x2);
+    const uint32_t s7_1 = lop3<0xe5>(s7_0, x5, x3);
+    const uint32_t s7_2 = lop3<0x9a>(x1, s7_1, x4);
+    const uint32_t s7_3 = lop3<0x61>(x1, x4, x3);
+    const uint32_t s7_4 = lop3<0x4d>(s7_3, s7_0, x3);
+    const uint32_t s7_5 = lop3<0x8a>(s7_4, x4, x0);
+    const uint32_t s7_6 = lop3<0x69>(s7_5, s7_3, x2);
+    const uint32_t s7_7 = lop3<0x94>(s7_2, s7_6, x5);
+    const uint32_t s7_8 = lop3<0x6a>(x0, s7_7, s7_4);
+    const uint32_t s7_9 = lop3<0xb3>(s7_8, s7_6, x5);
+    const uint32_t s7_10 = lop3<0xb2>(s7_9, s7_2, s7_4);
+    const uint32_t s7_11 = lop3<0x3e>(s7_10, x1, x5);
+    const uint32_t s7_12 = lop3<0x69>(x0, s7_8, s7_2);
+    T[14] = lop3<0x96>(T[14], s7_12, kc.z);
+    const uint32_t s7_13 = lop3<0x39>(s7_11, s7_6, s7_5);
+    const uint32_t s7_14 = lop3<0x69>(s7_13, s7_8, x5);
+    T[26] = lop3<0x96>(T[26], s7_14, kc.y);
+    const uint32_t s7_15 = lop3<0xa6>(s7_14, s7_5, x1);
+    const uint32_t s7_16 = lop3<0x69>(s7_15, s7_10, x0);
+    const uint32_t s7_17 = lop3<0x74>(s7_16, x5, s7_6);
+    T[4] = lop3<0x69>(T[4], s7_17, kc.x);
+    const uint32_t s7_18 = lop3<0xe4>(s7_16, s7_6, x5);
+    T[20] = lop3<0x69>(T[20], s7_18, kc.w);
     }
 }
 
