@@ -48,6 +48,12 @@ constexpr uint64_t kMixedMinBlocks = 8 * 1024;
 // scalar rounds finish far sooner than a bitsliced tile, and a bitsliced tile
 // would spend its full 1024-block work on them anyway.
 constexpr uint64_t kSplitBlocks = 512;
+// From this many blocks of medium messages their pieces are slices of mixed-key
+// tiles instead: a tile's latency (60 us) then is no longer than the scalar
+// items' time, and the blocks cost a third of the logic operations.
+// 4096 records of 64 B to 4 KiB through a context 909 -> 861 us, the 4096-message
+// batch 3482 -> 3461 us, the server's closed loop 391 -> 402 GB/s.
+constexpr uint64_t kMixedSplitBlocks = 128 * 1024;
 constexpr uint64_t kSoloChainBlocks = 512;                // longer CBC-enc chains: one per warp
 // What the choice for shorter chains weighs, in ns: a block of a chain that a
 // warp walks alone (one such chain per SM sub-partition at a time), a block of
@@ -330,10 +336,10 @@ __device__ __noinline__ void batch_scalar_item(const BatchParams& p, uint2 item,
 // Lane `lane` of slice sl: its message (index into msgs) and block, or false.
 __device__ __forceinline__ bool mixed_slot(const BatchParams& p, const MSlice& sl, uint32_t lane,
                                            uint32_t* msg, uint32_t* blk) {
-    if (lane >= sl.nvalid) return false;
+    if (lane >= (sl.nvalid & 63u)) return false;
     const uint32_t upto = sl.starts & (0xFFFFFFFFu >> (31u - lane));  // starts at lanes <= lane
     *msg = p.m_list[sl.msg0 + (uint32_t)__popc(upto) - 1u];
-    *blk = lane - (31u - (uint32_t)__clz(upto));
+    *blk = lane - (31u - (uint32_t)__clz(upto)) + (sl.nvalid >> 6);
     return true;
 }
 
@@ -422,16 +428,9 @@ __device__ __forceinline__ void stamp_warp_done(const BatchParams& p, uint32_t l
     }
 }
 
-// Programmatic dependent launch: the persistent kernel starts once every CTA of
-// the mixed-key kernel runs or has ended, and its warps wait for that kernel to
-// complete before they leave, so the stream's later work is ordered after both.
-__device__ __forceinline__ void launch_dependents() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-__device__ __forceinline__ void wait_for_primary() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-
+// The persistent kernel starts once every CTA of the mixed-key kernel runs or
+// has ended, and its warps wait for that kernel to complete before they leave,
+// so the stream's later work is ordered after both.
 __global__ void __launch_bounds__(256, 2) tdes_batch_mixed_kernel(BatchParams p) {
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     launch_dependents();  // the persistent kernel (other messages) runs beside this one
@@ -699,7 +698,10 @@ void build_plan(const tdes_desc_t* descs, uint32_t count, uint32_t key_count, in
     h->kind_bytes[mixed ? 1 : 2] += 8 * small_blocks;
     for (uint32_t mi : c_list) h->kind_bytes[3] += 8 * msgs[mi].nblocks;
     for (uint32_t mi : b_msg) h->kind_bytes[0] += 8 * msgs[mi].nblocks;
-    for (const SPiece& pc : split) h->kind_bytes[2] += 8ull * pc.n;
+    uint64_t split_blocks = 0;
+    for (const SPiece& pc : split) split_blocks += pc.n;
+    const bool mixed_split = split_blocks >= kMixedSplitBlocks;
+    h->kind_bytes[mixed_split ? 1 : 2] += 8 * split_blocks;
     for (const DirectMsg& m : h->direct) h->kind_bytes[4] += 8 * m.nblocks;
     if (mixed) {
         auto keydir = [&](uint32_t mi) {
@@ -726,10 +728,20 @@ void build_plan(const tdes_desc_t* descs, uint32_t count, uint32_t key_count, in
             m_list.push_back(mi);
         }
         if (open) m_slices.push_back(cur);
-        while (m_slices.size() % 32) m_slices.push_back({0u, 0u, 0u, 0u});  // empty slices
-        h->n_m_tiles = (uint32_t)(m_slices.size() / 32);
         s_list.clear();
     }
+    if (mixed_split) {  // a slice per piece, which needs no order of keys
+        for (const SPiece& pc : split) {
+            const uint32_t mode = msgs[pc.msg].mode;
+            const uint32_t dir = mode == TDES_MODE_ECB_DECRYPT || mode == TDES_MODE_CBC_DECRYPT;
+            m_slices.push_back({(uint32_t)m_list.size(), 1u, pc.n | pc.first << 6,
+                                (msgs[pc.msg].key << 1) | dir});
+            m_list.push_back(pc.msg);
+        }
+        split.clear();
+    }
+    while (m_slices.size() % 32) m_slices.push_back({0u, 0u, 0u, 0u});  // empty slices
+    h->n_m_tiles = (uint32_t)(m_slices.size() / 32);
     // S items: whole small messages (unless in mixed-key tiles) and the
     // pieces of medium ones, packed in order up to 32 blocks per item
     for (uint32_t mi : s_list) pieces.push_back({mi, 0u, (uint32_t)msgs[mi].nblocks, 0u});
@@ -899,22 +911,11 @@ cudaError_t enqueue_batch(const BatchParams& p_in, uint64_t total_items, bool ne
                                              (p.n_c_solo + 3) / 4);
     const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min(want, max_ctas));
     const bool solo = p.n_c_solo != 0, compact = shape.round_form == 1;
-    cudaLaunchAttribute beside = {};
-    beside.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    beside.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = 32 * warps;
-    cfg.dynamicSmemBytes = dyn_smem;
-    cfg.stream = s;
-    cfg.attrs = &beside;
-    cfg.numAttrs = p.n_m_tiles ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg,
-                              solo ? (compact ? tdes_batch_kernel<true, true>
-                                              : tdes_batch_kernel<true, false>)
-                                   : (compact ? tdes_batch_kernel<false, true>
-                                              : tdes_batch_kernel<false, false>),
-                              p);
+    return launch_kernel(solo ? (compact ? tdes_batch_kernel<true, true>
+                                         : tdes_batch_kernel<true, false>)
+                              : (compact ? tdes_batch_kernel<false, true>
+                                         : tdes_batch_kernel<false, false>),
+                         grid, 32 * warps, dyn_smem, s, p.n_m_tiles != 0, p);
 }
 
 cudaError_t enqueue_direct(const std::vector<DirectMsg>& direct, const tdes_keytable* kt,
@@ -928,15 +929,20 @@ cudaError_t enqueue_direct(const std::vector<DirectMsg>& direct, const tdes_keyt
         const bool vec16 = ((reinterpret_cast<uintptr_t>(m.in) | reinterpret_cast<uintptr_t>(m.out)) &
                             15u) == 0;
         const uint64_t ntiles = (m.nblocks + kTileBlocks - 1) / kTileBlocks;
+        auto geo = [&](int kernel) {
+            Geometry g = geometry_for(ntiles, kernel, device);
+            g.overlap = false;
+            return g;
+        };
         if (m.mode == TDES_MODE_CTR) {
             e = launch_ctr(tab, chunks, m.stages, (uint32_t)(m.iv >> 32), (uint32_t)m.iv, m.in, m.out,
-                           m.nblocks, vec16, geometry_for(ntiles, kCtr, device), s);
+                           m.nblocks, vec16, geo(kCtr), s);
         } else if (m.mode == TDES_MODE_CBC_DECRYPT) {
             e = launch_cbc_dec(tab, chunks, m.stages, m.iv, m.in, m.out, m.nblocks, nullptr, vec16,
-                               geometry_for(ntiles, kCbcDec, device), s);
+                               geo(kCbcDec), s);
         } else {
             e = launch_ecb(tab, chunks, m.stages, m.in, m.out, m.nblocks, vec16,
-                           geometry_for(ntiles, kEcb, device), s);
+                           geo(kEcb), s);
         }
         if (e != cudaSuccess) return e;
     }

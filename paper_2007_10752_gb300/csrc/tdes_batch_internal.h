@@ -29,11 +29,12 @@ constexpr int kChainSlots = 1024;  // SM sub-partitions tracked for C items (4 p
 constexpr int kCounterBytes = 32 + 4 * kChainSlots;
 
 // One slice (bit position) of a mixed-key tile: up to 32 blocks of small
-// messages under one key and direction, one block per lane.
+// messages, or one piece of a medium one, under one key and direction, one
+// block per lane.
 struct MSlice {
     uint32_t msg0;    // first of the slice's messages in m_list
     uint32_t starts;  // bit l set where a message begins at lane l
-    uint32_t nvalid;  // lanes [0, nvalid) hold blocks
+    uint32_t nvalid;  // lanes [0, nvalid % 64) hold blocks; nvalid / 64: a piece's first block
     uint32_t keydir;  // key << 1 | direction (1: decryption table)
 };
 

