@@ -85,6 +85,12 @@ struct Pending {
 // a warp walks at about a microsecond per block.  A batch completes as a
 // whole, so requests batched with it would wait for it: it gets a batch of
 // its own instead.
+// A batch takes requests until their input and output pass this many bytes: the
+// device starts on the first of a burst while the next is planned, and the
+// batches fill each other's tails.  1024 requests of the serving mix at once
+// 2156 -> 1902 us, closed loop 401.7 -> 405.7 GB/s, p99 at 330 GB/s 0.51 -> 0.38
+// ms, p50 and p99 below 180 GB/s unchanged; with four times as much 1929 us.
+constexpr uint64_t kBatchCost = 32ull << 20;
 constexpr uint64_t kLoneChainBlocks = 512;
 bool lone_request(const tdes_desc_t& d) {
     return d.mode == TDES_MODE_CBC_ENCRYPT && d.nbytes / 8 > kLoneChainBlocks;
@@ -280,7 +286,7 @@ struct tdes_server {
                 if (queued.load(std::memory_order_acquire) == 0) break;  // nothing to take
                 {
                     std::lock_guard<std::mutex> lock(mu);
-                    while (!queue.empty() && take.size() < cfg.max_batch &&
+                    while (!queue.empty() && take.size() < cfg.max_batch && cost < kBatchCost &&
                            admitted + cost + queue.front().cost <= cfg.budget_bytes) {
                         const bool alone = queue.front().alone;
                         if (alone && !take.empty()) break;  // it starts the next batch
