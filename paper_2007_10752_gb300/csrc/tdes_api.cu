@@ -129,8 +129,10 @@ Geometry geometry_for(uint64_t ntiles, int kernel_id, int device) {
     const DeviceInfo* d = device_info(device);
     const int sms = d ? d->sms : 1;
     const int per_sm = d ? d->ctas_per_sm[kernel_id] : 1;
-    if (ntiles <= 4ull * sms) return {(int)(ntiles ? ntiles : 1), 32, sms};
-    return {sms * per_sm, 32 * kWideWarps, sms};
+    // one-warp CTAs wait for the kernel before: started beside it they would
+    // take the places it leaves, unevenly over the sub-partitions
+    if (ntiles <= 4ull * sms) return {(int)(ntiles ? ntiles : 1), 32, sms, false};
+    return {sms * per_sm, 32 * kWideWarps, sms, true};
 }
 
 }  // namespace tdes
@@ -389,7 +391,8 @@ int tdes_ecb_crypt_host(const tdes_ks_t* ks, int decrypt, const void* host_in, v
         what = "ECB kernel";
         if (e == cudaSuccess) e = cudaStreamWaitEvent(scomp, ev_in[b], 0);
         if (e == cudaSuccess) {
-            const tdes::Geometry g = tdes::geometry_for(ntiles, tdes::kEcb, ks->device);
+            tdes::Geometry g = tdes::geometry_for(ntiles, tdes::kEcb, ks->device);
+            g.overlap = false;  // each chunk's kernel waits for its copy anyway
             e = tdes::launch_ecb(ks->tab[decrypt ? 1 : 0], ks->chunk[decrypt ? 1 : 0], ks->stages, buf, buf, nblocks, true,
                                  g, scomp);
         }

@@ -129,23 +129,26 @@ __device__ __forceinline__ uint32_t bswap32(uint32_t x) { return __byte_perm(x, 
 // ------------------------------------------------ first tile of a warp, tail
 // Tile of a warp's first pass (the later ones follow a stride of all warps).
 // The passes run CTA by CTA within a rank, and a CTA ranks its warps by SM
-// sub-partition, the first CTA of an SM from sub-partition 0 and the second
-// from 2, so that a last pass with fewer tiles than warps loads every
-// sub-partition alike: a tile alone on one takes 17 us, four together 46 us.
+// sub-partition, from 0 in the CTA that holds the SM's warp slot 0 and from 2 in
+// the other, so that a last pass with fewer tiles than warps loads every
+// sub-partition alike: a tile alone on one takes 17 us, four together 44 us.
 // (Consecutive tiles per CTA put the 84 last tiles of 1300 on 11 SMs: 50.6
-// against 35.4 us.)  %warpid is only a hint: any values give each warp a rank
-// of its own.  publish_rank before a barrier, first_tile after it.
-__device__ __forceinline__ void publish_rank(uint32_t* order) {
+// against 35.4 us.  In a kernel that starts beside the one before, slots are
+// taken as they come free, and 700 tiles take 30 instead of 27 us.)  %warpid is only a hint: any values give each warp a rank
+// of its own.  publish_slot before a barrier, first_tile after it.
+__device__ __forceinline__ void publish_slot(uint32_t* slots) {
     uint32_t slot;
     asm("mov.u32 %0, %%warpid;" : "=r"(slot));
-    if ((threadIdx.x & 31u) == 0)
-        order[threadIdx.x >> 5] =
-            8u * ((slot & 4u) | ((slot ^ (slot >> 2 & 2u)) & 3u)) + (threadIdx.x >> 5);
+    if ((threadIdx.x & 31u) == 0) slots[threadIdx.x >> 5] = slot;
 }
-__device__ __forceinline__ uint32_t first_tile(const uint32_t* order) {
-    const uint32_t warps = blockDim.x >> 5, mine = order[threadIdx.x >> 5];
+__device__ __forceinline__ uint32_t first_tile(const uint32_t* slots) {
+    const uint32_t warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
+    uint32_t lowest = slots[0];
+    for (uint32_t w = 1; w < warps; ++w) lowest = min(lowest, slots[w]);
+    const uint32_t turn = lowest ? 2u : 0u;
+    const uint32_t mine = (slots[warp] ^ turn) * kWideWarps + warp;
     uint32_t rank = 0;
-    for (uint32_t w = 0; w < warps; ++w) rank += order[w] < mine;
+    for (uint32_t w = 0; w < warps; ++w) rank += (slots[w] ^ turn) * kWideWarps + w < mine;
     return rank * gridDim.x + blockIdx.x;
 }
 
@@ -204,10 +207,12 @@ tdes_ecb_kernel(const uint32_t* __restrict__ table, const uint8_t* in, uint8_t* 
                 uint64_t nblocks, Tail tail) {
     __shared__ __align__(16) uint32_t tab[table_words<STAGES>()];
     extern __shared__ __align__(16) uint4 ecb_data[];  // kCtrWarpBytes per warp (VEC only)
-    __shared__ uint32_t order[kWideWarps];
+    __shared__ uint32_t slots[kWideWarps];
+    launch_dependents();
     stage_table<STAGES>(tab, table);
-    publish_rank(order);
+    publish_slot(slots);
     __syncthreads();
+    wait_for_primary();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warps = blockDim.x >> 5;
     uint4* wbuf = ecb_data + (threadIdx.x >> 5) * (kCtrWarpBytes / 16);
@@ -215,7 +220,7 @@ tdes_ecb_kernel(const uint32_t* __restrict__ table, const uint8_t* in, uint8_t* 
     const uint32_t ntiles = (uint32_t)((nblocks + kTileBlocks - 1) / kTileBlocks);
     const uint32_t nfull = (uint32_t)(nblocks / kTileBlocks);  // tiles [0, nfull) are full
     const uint32_t stride = gridDim.x * warps;
-    uint32_t t = first_tile(order);
+    uint32_t t = first_tile(slots);
     if (VEC && t < nfull) {
         const uint4* p = reinterpret_cast<const uint4*>(in) + (uint64_t)t * (kTileBlocks / 2) + lane;
 #pragma unroll
@@ -308,15 +313,11 @@ static uint64_t tail_split(int stages, bool vec16, Geometry g, const uint8_t* ch
 }
 
 template <int STAGES>
-static void ecb_launch(const uint32_t* tab, const void* in, void* out, uint64_t nblocks,
+static cudaError_t ecb_launch(const uint32_t* tab, const void* in, void* out, uint64_t nblocks,
                        bool vec16, Geometry g, Tail tail, cudaStream_t s) {
-    if (vec16)
-        tdes_ecb_kernel<true, STAGES>
-            <<<g.grid, g.threads, (size_t)(g.threads / 32) * kCtrWarpBytes, s>>>(
-                tab, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out), nblocks, tail);
-    else
-        tdes_ecb_kernel<false, STAGES><<<g.grid, g.threads, 0, s>>>(
-            tab, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out), nblocks, tail);
+    return launch_kernel(vec16 ? tdes_ecb_kernel<true, STAGES> : tdes_ecb_kernel<false, STAGES>, g.grid,
+                  g.threads, vec16 ? (size_t)(g.threads / 32) * kCtrWarpBytes : 0, s, g.overlap, tab,
+                  static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out), nblocks, tail);
 }
 
 cudaError_t launch_ecb(const uint32_t* tab, const uint8_t* chunks, int stages, const void* in,
@@ -325,11 +326,8 @@ cudaError_t launch_ecb(const uint32_t* tab, const uint8_t* chunks, int stages, c
     if (e != cudaSuccess) return e;
     Tail tail;
     nblocks = tail_split(stages, vec16, g, chunks, nblocks, &tail);
-    if (stages == 1)
-        ecb_launch<1>(tab, in, out, nblocks, vec16, g, tail, s);
-    else
-        ecb_launch<3>(tab, in, out, nblocks, vec16, g, tail, s);
-    return cudaGetLastError();
+    return stages == 1 ? ecb_launch<1>(tab, in, out, nblocks, vec16, g, tail, s)
+                       : ecb_launch<3>(tab, in, out, nblocks, vec16, g, tail, s);
 }
 
 // ------------------------------------------------------------------- CTR
@@ -344,10 +342,12 @@ tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr
                 const uint8_t* in, uint8_t* out, uint64_t nblocks, Tail tail) {
     __shared__ __align__(16) uint32_t tab[table_words<STAGES>()];
     extern __shared__ __align__(16) uint4 ctr_data[];  // kCtrWarpBytes per warp
-    __shared__ uint32_t order[kWideWarps];
+    __shared__ uint32_t slots[kWideWarps];
+    launch_dependents();
     stage_table<STAGES>(tab, table);
-    publish_rank(order);
+    publish_slot(slots);
     __syncthreads();
+    wait_for_primary();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warps = blockDim.x >> 5;
     uint4* wbuf = ctr_data + (threadIdx.x >> 5) * (kCtrWarpBytes / 16);
@@ -357,7 +357,7 @@ tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr
     // Tile indices fit 32 bits: the host caps a call below 2^31 tiles.
     using Idx = typename std::conditional<VEC, uint64_t, uint32_t>::type;
     const Idx ntiles = (Idx)((nblocks + kTileBlocks - 1) / kTileBlocks);
-    for (Idx t = first_tile(order); t < ntiles; t += (Idx)gridDim.x * warps) {
+    for (Idx t = first_tile(slots); t < ntiles; t += (Idx)gridDim.x * warps) {
         const uint64_t b0 = (uint64_t)t * kTileBlocks;
         const bool full = VEC && b0 + kTileBlocks <= nblocks;
         if (full) {  // each lane copies, and later reads back, only its own 16 x 16 bytes
@@ -428,18 +428,13 @@ tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr
 }
 
 template <int STAGES>
-static void ctr_launch(const uint32_t* tab_enc, uint32_t nonce, uint32_t ctr0, const void* in,
+static cudaError_t ctr_launch(const uint32_t* tab_enc, uint32_t nonce, uint32_t ctr0, const void* in,
                        void* out, uint64_t nblocks, bool vec16, Geometry g, Tail tail,
                        cudaStream_t s) {
     const size_t dyn = (size_t)(g.threads / 32) * kCtrWarpBytes;
-    if (vec16)
-        tdes_ctr_kernel<true, STAGES><<<g.grid, g.threads, dyn, s>>>(
-            tab_enc, nonce, ctr0, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out),
-            nblocks, tail);
-    else
-        tdes_ctr_kernel<false, STAGES><<<g.grid, g.threads, dyn, s>>>(
-            tab_enc, nonce, ctr0, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out),
-            nblocks, tail);
+    return launch_kernel(vec16 ? tdes_ctr_kernel<true, STAGES> : tdes_ctr_kernel<false, STAGES>, g.grid,
+                  g.threads, dyn, s, g.overlap, tab_enc, nonce, ctr0,
+                  static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out), nblocks, tail);
 }
 
 cudaError_t launch_ctr(const uint32_t* tab_enc, const uint8_t* chunks, int stages, uint32_t nonce,
@@ -449,11 +444,8 @@ cudaError_t launch_ctr(const uint32_t* tab_enc, const uint8_t* chunks, int stage
     if (e != cudaSuccess) return e;
     Tail tail;
     nblocks = tail_split(stages, vec16, g, chunks, nblocks, &tail);
-    if (stages == 1)
-        ctr_launch<1>(tab_enc, nonce, ctr0, in, out, nblocks, vec16, g, tail, s);
-    else
-        ctr_launch<3>(tab_enc, nonce, ctr0, in, out, nblocks, vec16, g, tail, s);
-    return cudaGetLastError();
+    return stages == 1 ? ctr_launch<1>(tab_enc, nonce, ctr0, in, out, nblocks, vec16, g, tail, s)
+                       : ctr_launch<3>(tab_enc, nonce, ctr0, in, out, nblocks, vec16, g, tail, s);
 }
 
 // --------------------------------------------------------------- CBC decrypt
@@ -484,10 +476,12 @@ tdes_cbc_dec_kernel(const uint32_t* __restrict__ table, uint64_t iv, const uint8
                     Tail tail) {
     __shared__ __align__(16) uint32_t tab[table_words<STAGES>()];
     extern __shared__ __align__(16) uint4 cbc_data[];  // kCtrWarpBytes per warp (VEC only)
-    __shared__ uint32_t order[kWideWarps];
+    __shared__ uint32_t slots[kWideWarps];
+    launch_dependents();
     stage_table<STAGES>(tab, table);
-    publish_rank(order);
+    publish_slot(slots);
     __syncthreads();
+    wait_for_primary();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warps = blockDim.x >> 5;
     uint4* wbuf = cbc_data + (threadIdx.x >> 5) * (kCtrWarpBytes / 16);
@@ -497,7 +491,7 @@ tdes_cbc_dec_kernel(const uint32_t* __restrict__ table, uint64_t iv, const uint8
     const uint32_t stride = gridDim.x * warps;
     const uint2 ivw = make_uint2(bswap32((uint32_t)(iv >> 32)), bswap32((uint32_t)iv));
     const uint2* c = reinterpret_cast<const uint2*>(in);
-    uint32_t t = first_tile(order);
+    uint32_t t = first_tile(slots);
     if (VEC && t < nfull) {  // full tiles are prefetched one ahead, as in ECB
         const uint4* p = reinterpret_cast<const uint4*>(in) + (uint64_t)t * (kTileBlocks / 2) + lane;
 #pragma unroll
@@ -564,18 +558,13 @@ tdes_cbc_dec_kernel(const uint32_t* __restrict__ table, uint64_t iv, const uint8
 }
 
 template <int STAGES>
-static void cbc_dec_launch(const uint32_t* tab_dec, uint64_t iv, const void* in, void* out,
+static cudaError_t cbc_dec_launch(const uint32_t* tab_dec, uint64_t iv, const void* in, void* out,
                            uint64_t nblocks, const uint64_t* halo, bool vec16, Geometry g,
                            Tail tail, cudaStream_t s) {
-    if (vec16)
-        tdes_cbc_dec_kernel<true, STAGES>
-            <<<g.grid, g.threads, (size_t)(g.threads / 32) * kCtrWarpBytes, s>>>(
-                tab_dec, iv, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out),
-                nblocks, halo, tail);
-    else
-        tdes_cbc_dec_kernel<false, STAGES><<<g.grid, g.threads, 0, s>>>(
-            tab_dec, iv, static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out), nblocks,
-            halo, tail);
+    return launch_kernel(vec16 ? tdes_cbc_dec_kernel<true, STAGES> : tdes_cbc_dec_kernel<false, STAGES>,
+                  g.grid, g.threads, vec16 ? (size_t)(g.threads / 32) * kCtrWarpBytes : 0, s,
+                  g.overlap, tab_dec, iv, static_cast<const uint8_t*>(in),
+                  static_cast<uint8_t*>(out), nblocks, halo, tail);
 }
 
 cudaError_t launch_cbc_dec(const uint32_t* tab_dec, const uint8_t* chunks, int stages, uint64_t iv,
@@ -585,11 +574,9 @@ cudaError_t launch_cbc_dec(const uint32_t* tab_dec, const uint8_t* chunks, int s
     if (e != cudaSuccess) return e;
     Tail tail;  // in place a tail block's predecessor may be overwritten before it is read
     nblocks = tail_split(stages, vec16, g, in == out ? nullptr : chunks, nblocks, &tail);
-    if (stages == 1)
-        cbc_dec_launch<1>(tab_dec, iv, in, out, nblocks, halo, vec16, g, tail, s);
-    else
-        cbc_dec_launch<3>(tab_dec, iv, in, out, nblocks, halo, vec16, g, tail, s);
-    return cudaGetLastError();
+    return stages == 1
+               ? cbc_dec_launch<1>(tab_dec, iv, in, out, nblocks, halo, vec16, g, tail, s)
+               : cbc_dec_launch<3>(tab_dec, iv, in, out, nblocks, halo, vec16, g, tail, s);
 }
 
 // --------------------------------------------------------------- CBC encrypt
@@ -603,24 +590,22 @@ __global__ void __launch_bounds__(kChainThreads)
 tdes_cbc_enc_kernel(const uint8_t* __restrict__ chunks_g, uint64_t iv, const uint8_t* in,
                     uint8_t* out, uint64_t nblocks) {
     __shared__ uint2 tab[32 * ROUNDS];
+    launch_dependents();
     const uint32_t lane = threadIdx.x & 31u;
     const ChainLane c = {kLaneSbox[lane][0], kLaneSbox[lane][1], kLaneSbox[lane][2],
                          kLaneSbox[lane][3]};
     chain_tables<ROUNDS>(tab, c, chunks_g, lane, threadIdx.x >> 5, blockDim.x >> 5);
     __syncthreads();
     if (threadIdx.x >= 32) return;
+    wait_for_primary();
     chain_walk<ROUNDS>(in, out, nblocks, iv, c.rot, lane, tab);
 }
 
 cudaError_t launch_cbc_enc(const uint8_t* chunk_enc, int stages, uint64_t iv, const void* in,
                            void* out, uint64_t nblocks, cudaStream_t s) {
-    if (stages == 1)
-        tdes_cbc_enc_kernel<16><<<1, kChainThreads, 0, s>>>(chunk_enc, iv, static_cast<const uint8_t*>(in),
-                                                 static_cast<uint8_t*>(out), nblocks);
-    else
-        tdes_cbc_enc_kernel<48><<<1, kChainThreads, 0, s>>>(chunk_enc, iv, static_cast<const uint8_t*>(in),
-                                                 static_cast<uint8_t*>(out), nblocks);
-    return cudaGetLastError();
+    return launch_kernel(stages == 1 ? tdes_cbc_enc_kernel<16> : tdes_cbc_enc_kernel<48>, 1,
+                         kChainThreads, 0, s, true, chunk_enc, iv, static_cast<const uint8_t*>(in),
+                         static_cast<uint8_t*>(out), nblocks);
 }
 
 // ------------------------------------------------------------- occupancy
