@@ -57,18 +57,20 @@ constexpr int kTileWarpBytes = kUniTableBytes + kTileSlots * 4;
 // one held block per chain (25 KB; one CTA per SM of 8 warps for mixed-key
 // chains, 9 for single-key tiles)
 constexpr int kChainWarpBytes = kUniTableBytes + 32 * 32 * 4 + 32 * 32 * 8;
-// Mixed-key CBC-encryption slices: 12 warps per CTA, one CTA per SM, each
-// warp with its table and its chains' message indices in shared memory
-// (17 KB) and its held blocks in a slab of global scratch (8 KB per warp).
-constexpr int kMixedChainWarps = 12;
+// Mixed-key CBC-encryption slices: 6 warps per CTA, each warp with its table
+// and its chains' message indices in shared memory (17 KB) and its held blocks
+// in a slab of global scratch (8 KB per warp).  Two launches of a CTA per SM
+// make 12 warps of them, and a CTA fits beside a tile kernel's.
+constexpr int kMixedChainWarps = 6;
 constexpr int kMixedChainWarpBytes = kUniTableBytes + 32 * 32 * 4;
 constexpr int kMaxChainCtas = 256;  // the kernel's grid: min(SMs, this)
 // sm_103a shared memory: 228 KB per SM, 1 KB of it reserved per resident CTA,
 // so a CTA may take at most 227 KB
 constexpr int kSmemPerSm = 228 * 1024, kSmemReservedPerCta = 1024;
 static_assert(kKeyChainWarps * kChainWarpBytes + kSmemReservedPerCta <= kSmemPerSm, "single-key chain CTA");
-static_assert(kMixedChainWarps * kMixedChainWarpBytes + kSmemReservedPerCta <= kSmemPerSm,
-              "mixed-key chain CTA");
+static_assert(kMixedChainWarps * kMixedChainWarpBytes + kUniWarps * kMixedWarpBytes +
+                      2 * kSmemReservedPerCta <= kSmemPerSm,
+              "a mixed-key chain CTA beside a tile CTA");
 static_assert(2 * (kUniWarps * kTileWarpBytes + kSmemReservedPerCta) <= kSmemPerSm, "two tile CTAs per SM");
 static_assert(2 * (kUniWarps * kMixedWarpBytes + kSmemReservedPerCta) <= kSmemPerSm,
               "two mixed-key CTAs per SM");
@@ -83,7 +85,8 @@ struct UniHeader {
     uint32_t slices[2];          // mixed-key slices: [0] modes 0-3 from slice 0,
     uint32_t slice2_base;        //   [1] CBC encryption from slice2_base (a multiple of 32)
     uint32_t kind_tiles[5];      // single-key tiles of kind k: [kind_tiles[k], kind_tiles[k + 1])
-    uint32_t pad[4];
+    uint32_t chain_next;         // next tile of 32 CBC-encryption slices to claim
+    uint32_t pad[3];
 };
 static_assert(sizeof(UniHeader) == 64, "header layout");
 
@@ -357,6 +360,14 @@ __global__ void uni_scatter_kernel(UniParams p) {
         base = __shfl_sync(act, base, leader);
         if (g != ~0u) p.order[base + __popc(peers & ((1u << lane) - 1u))] = (uint32_t)i;
     }
+}
+
+// The work kernels share no messages, so each starts once every CTA of the one
+// before runs or has ended (programmatic dependent launch), and its CTAs take
+// the places that the other's leave.  The first CTA of each waits for the
+// kernel before to complete, so the last kernel's end is the call's.
+__device__ __forceinline__ void first_cta_waits() {
+    if (blockIdx.x == 0) wait_for_primary();
 }
 
 extern __shared__ __align__(16) uint8_t uni_smem[];  // a slice per warp (kTileWarpBytes, ...)
@@ -683,13 +694,15 @@ __device__ __forceinline__ void uni_chain_tile(const UniParams& p, uint32_t t, u
 template <int KIND, bool VEC16>
 __global__ void __launch_bounds__(KIND == kKindCbcEnc ? 32 * kKeyChainWarps : 32 * kUniWarps,
                                   KIND == kKindCbcEnc ? 1 : 2) uni_tile_kernel(UniParams p) {
+    launch_dependents();
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     uint32_t* wtab = reinterpret_cast<uint32_t*>(
         uni_smem + (size_t)warp * (KIND == kKindCbcEnc ? kChainWarpBytes : kTileWarpBytes));
     const uint32_t first = p.hdr->kind_tiles[KIND];
     const uint32_t n = p.hdr->kind_tiles[KIND + 1] - first;
     const uint32_t nw = blockDim.x >> 5;
-    const uint32_t W = gridDim.x * nw, w = blockIdx.x * nw + warp;
+    // run by run over the CTAs, so that few tiles spread over the SMs
+    const uint32_t W = gridDim.x * nw, w = warp * gridDim.x + blockIdx.x;
     const uint32_t per = n / W, extra = n % W;
     const uint32_t a = w * per + min(w, extra), b = a + per + (w < extra ? 1u : 0u);
     uint32_t staged = ~0u;
@@ -711,6 +724,7 @@ __global__ void __launch_bounds__(KIND == kKindCbcEnc ? 32 * kKeyChainWarps : 32
         else
             uni_block_tile<KIND, VEC16>(p, t, wtab, wtab + TDES_TABLE_WORDS, lane, one_pass);
     }
+    first_cta_waits();
 }
 
 // Mixed-key tiles: slice s of tile t is slice first + 32 t + s; lane s works
@@ -718,9 +732,12 @@ __global__ void __launch_bounds__(KIND == kKindCbcEnc ? 32 * kKeyChainWarps : 32
 // key's packed table row, and a transpose across the lanes builds the tile's
 // table (bit s of every word: slice s's key and direction).  Slices differ
 // in mode, but each slice's mode is the same in every lane.
+// Chain tiles are claimed from a counter, by both launches of the kernel (late:
+// the second).
 template <bool CHAIN>
-__global__ void __launch_bounds__(CHAIN ? 32 * kMixedChainWarps : 32 * kUniWarps, CHAIN ? 1 : 2)
-    uni_mixed_kernel(UniParams p) {
+__global__ void __launch_bounds__(CHAIN ? 32 * kMixedChainWarps : 32 * kUniWarps, 2)
+    uni_mixed_kernel(UniParams p, uint32_t late) {
+    launch_dependents();
     constexpr uint32_t kWarps = CHAIN ? kMixedChainWarps : kUniWarps;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     uint32_t* wtab = reinterpret_cast<uint32_t*>(
@@ -729,7 +746,13 @@ __global__ void __launch_bounds__(CHAIN ? 32 * kMixedChainWarps : 32 * kUniWarps
     const uint32_t ns = CHAIN ? p.hdr->slices[1] : p.hdr->slices[0];
     const uint32_t ntiles = (ns + 31u) / 32u;
     const uint32_t W = gridDim.x * kWarps;
-    for (uint32_t t = blockIdx.x * kWarps + warp; t < ntiles; t += W) {
+    auto claim = [&](uint32_t t) {  // the tile after t
+        if (!CHAIN) return t + W;
+        uint32_t c = 0;
+        if (lane == 0) c = atomicAdd(&p.hdr->chain_next, 1u);
+        return __shfl_sync(0xFFFFFFFFu, c, 0);
+    };
+    for (uint32_t t = CHAIN ? claim(0u) : warp * gridDim.x + blockIdx.x; t < ntiles; t = claim(t)) {
         uint32_t pos = 0, cm = 0, kd = 0;  // cm: message count | mode << 8
         if (32u * t + lane < ns) {
             const uint32_t s = first + 32u * t + lane;
@@ -771,8 +794,8 @@ __global__ void __launch_bounds__(CHAIN ? 32 * kMixedChainWarps : 32 * kUniWarps
                 A1[s] = c.y;
             }
             uni_chain_passes<true>(p, A0, A1, wtab, widx,
-                                   p.held + (size_t)(blockIdx.x * kWarps + warp) * (32 * 32), lane,
-                                   false);
+                                   p.held + (size_t)((2u * blockIdx.x + late) * kWarps + warp) * (32 * 32),
+                                   lane, false);
         } else {
             // lane l holds block l % m of the slice's message l / m.  With at
             // most kSliceSlots messages a slice, each message's index (written
@@ -844,6 +867,7 @@ __global__ void __launch_bounds__(CHAIN ? 32 * kMixedChainWarps : 32 * kUniWarps
             __syncwarp();  // sidx and smode are rewritten by the next tile
         }
     }
+    first_cta_waits();
 }
 
 // ------------------------------------------------------------------- host
@@ -890,7 +914,7 @@ UniLayout layout_for(uint64_t n_msgs, uint32_t m, uint32_t n_keys) {
     L.o_part = L.o_sg + al256(L.max_slices * 4);
     L.o_base = L.o_part + al256((size_t)scan_blocks(n_keys) * sizeof(Sums));
     L.o_held = L.o_base + al256((size_t)scan_blocks(n_keys) * sizeof(Sums));
-    L.total = L.o_held + (size_t)kMaxChainCtas * kMixedChainWarps * 32 * 32 * sizeof(uint2);
+    L.total = L.o_held + (size_t)kMaxChainCtas * 2 * kMixedChainWarps * 32 * 32 * sizeof(uint2);
     return L;
 }
 
@@ -1054,38 +1078,45 @@ int tdes_uniform_crypt(const tdes_keytable_t* kt, const uint32_t* key_index, con
     }
     if (e == cudaSuccess) {
         what = "work kernels";
-        const dim3 g(work_grid), b(32 * kUniWarps);
-        if (vec16) {
-            uni_tile_kernel<kKindEcb, true><<<g, b, dyn, s>>>(p);
-            uni_tile_kernel<kKindCtr, true><<<g, b, dyn, s>>>(p);
-            uni_tile_kernel<kKindCbcDec, true><<<g, b, dyn, s>>>(p);
-        } else {
-            uni_tile_kernel<kKindEcb, false><<<g, b, dyn, s>>>(p);
-            uni_tile_kernel<kKindCtr, false><<<g, b, dyn, s>>>(p);
-            uni_tile_kernel<kKindCbcDec, false><<<g, b, dyn, s>>>(p);
-        }
-        uni_mixed_kernel<false><<<g, b, (size_t)kUniWarps * kMixedWarpBytes, s>>>(p);
-        // CBC-encryption chains: one CTA per SM, each warp with room for its
-        // chains' message indices (2^28 messages of 64 B: 75.2 -> 73.1 ms
-        // with the indices, alternating A/B runs) and its held blocks.  The
-        // single-key tiles keep both in shared memory, 9 warps per CTA (2^22
-        // single-key chains of 64 B: 1.60 -> 1.52 ms against 8).  The
-        // mixed-key slices keep the held blocks in their warp's slab of
-        // global scratch instead, which lets 12 warps fit (65.10 -> 64.65
-        // ms for 2^28 messages, against 8 warps with everything in shared
-        // memory; with the slab's accesses asking L2 to keep its lines,
-        // 64.20 ms); with the indices there too, 16 warps at 128 registers
-        // spilled 308 bytes and took 66.3 ms.  The single-key tiles with
-        // their held blocks in the slab at 12 warps were slower (2^22 chains
-        // under two keys: 1.71 -> 1.91 ms): with few keys a tile's chains lie
-        // close together, their data is mostly in L2 already, and the
-        // shared-memory held blocks' shorter latency counts for more.
-        const dim3 g1(geo.sms);
-        uni_tile_kernel<kKindCbcEnc, false><<<g1, dim3(32 * kKeyChainWarps),
-                                              (size_t)kKeyChainWarps * kChainWarpBytes, s>>>(p);
-        uni_mixed_kernel<true><<<dim3(std::min(geo.sms, kMaxChainCtas)), dim3(32 * kMixedChainWarps),
-                                 (size_t)kMixedChainWarps * kMixedChainWarpBytes, s>>>(p);
-        e = cudaGetLastError();
+        // CBC-encryption chains of mixed-key slices: two launches of a CTA per
+        // SM, the first before the tiles, with its CTAs beside theirs: alone the
+        // chains keep the logic pipe half busy.  In larger calls the tiles' traffic
+        // drives the chains' messages out of L2 between passes, and both launches
+        // come last (64 B: 256 MB 1187 us first, 1469 us last; 1 GB 4113 and 3910
+        // us; 128 B: 1 GB 3674 and 3810 us; 256 B: 1 GB 3429 and 4327 us; 16 B: 64
+        // MB 648 and 712 us, 128 MB 1215 and 1173 us).
+        // Their held blocks in a slab of global scratch, with accesses that ask
+        // L2 to keep its lines, beat 8 warps with everything in shared memory
+        // (2^28 messages of 64 B: 65.10 -> 64.20 ms); with the message indices
+        // there too, 16 warps at 128 registers spilled 308 bytes and took 66.3
+        // ms.  The single-key tiles of chains keep both in shared memory, 9
+        // warps per CTA (2^22 single-key chains: 1.60 -> 1.52 ms against 8; with
+        // the slab at 12 warps 1.91 ms: with few keys a tile's chains lie close
+        // together and their data is mostly in L2 already).
+        const unsigned chain_ctas = std::min(geo.sms, kMaxChainCtas);
+        const size_t dyn_mixed = (size_t)kUniWarps * kMixedWarpBytes;
+        const size_t dyn_chain = (size_t)kMixedChainWarps * kMixedChainWarpBytes;
+        const size_t dyn_key_chain = (size_t)kKeyChainWarps * kChainWarpBytes;
+        const bool chains_first = span <= (msg_bytes >= 32 ? msg_bytes << 23 : 64ull << 20);
+        bool first = true;
+        auto work = [&](unsigned ctas, int warps, size_t smem, auto kernel, auto... args) {
+            if (e == cudaSuccess)
+                e = launch_kernel(kernel, ctas, 32 * warps, smem, s, !first, args...);
+            first = false;
+        };
+        if (chains_first)
+            work(chain_ctas, kMixedChainWarps, dyn_chain, uni_mixed_kernel<true>, p, 0u);
+        work(work_grid, kUniWarps, dyn,
+             vec16 ? uni_tile_kernel<kKindEcb, true> : uni_tile_kernel<kKindEcb, false>, p);
+        work(work_grid, kUniWarps, dyn,
+             vec16 ? uni_tile_kernel<kKindCtr, true> : uni_tile_kernel<kKindCtr, false>, p);
+        work(work_grid, kUniWarps, dyn,
+             vec16 ? uni_tile_kernel<kKindCbcDec, true> : uni_tile_kernel<kKindCbcDec, false>, p);
+        work(work_grid, kUniWarps, dyn_mixed, uni_mixed_kernel<false>, p, 0u);
+        if (!chains_first)
+            work(chain_ctas, kMixedChainWarps, dyn_chain, uni_mixed_kernel<true>, p, 0u);
+        work(chain_ctas, kMixedChainWarps, dyn_chain, uni_mixed_kernel<true>, p, 1u);
+        work(geo.sms, kKeyChainWarps, dyn_key_chain, uni_tile_kernel<kKindCbcEnc, false>, p);
     }
     if (e == cudaSuccess && skipped != nullptr) {
         what = "copying the skipped count";
