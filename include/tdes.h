@@ -198,7 +198,8 @@ typedef struct {
     int ctas_per_sm;
     uint64_t bytes_per_mode[5];  /* payload bytes, indexed by TDES_MODE_* */
     uint64_t n_mixed_tiles;      /* bitsliced tiles of small messages under up to 32 keys
-                                    (batches with 8192 or more small-message blocks) */
+                                    (batches with 8192 or more small-message blocks, or
+                                    131072 or more blocks in messages of 33 to 512) */
     uint32_t n_direct_messages;  /* messages of 64 MiB or more (ECB, CTR, out-of-place CBC
                                     decryption) run by the single-key kernels */
     int tiles_per_claim;         /* tiles a warp claims at once (the automatic choice resolved) */

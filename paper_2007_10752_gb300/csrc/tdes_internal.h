@@ -79,7 +79,7 @@ struct Geometry {
     int grid;
     int threads;
     int sms;
-    bool overlap = true;  // launch_kernel
+    bool overlap;  // launch_kernel
 };
 
 // The blocks of a call that run one per thread after the kernel's tiles: n of
