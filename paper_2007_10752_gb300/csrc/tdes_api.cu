@@ -103,7 +103,7 @@ bool host_memory(const void* p) {
     return a.type == cudaMemoryTypeHost;
 }
 
-bool gpu_addressable(const void* p) {
+bool gpu_addressable(const void* p, bool* host) {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();  // clear the sticky-free error of the query
@@ -114,6 +114,7 @@ bool gpu_addressable(const void* p) {
         case cudaMemoryTypeManaged:
             return true;
         case cudaMemoryTypeHost:
+            if (host != nullptr) *host = true;
             return a.devicePointer == p;
         default:
             return false;

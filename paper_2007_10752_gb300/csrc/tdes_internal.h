@@ -23,8 +23,9 @@ void set_last_error(const char* msg);
 // True if the GPU can address `p` with the same pointer: device or managed
 // memory, or page-locked host memory mapped into the device address space
 // (what cudaHostAlloc gives on a unified-address system).  Pageable host
-// memory is refused: a kernel access to it could fault.
-bool gpu_addressable(const void* p);
+// memory is refused: a kernel access to it could fault.  Sets *host (where
+// given) for host memory and leaves it alone otherwise.
+bool gpu_addressable(const void* p, bool* host = nullptr);
 // True for page-locked host memory (whether or not it is mapped).
 bool host_memory(const void* p);
 

@@ -79,18 +79,22 @@ struct Pending {
     uint64_t cost;
     bool stage;  // host buffers, large enough to be staged through the device
     bool alone;  // a long serial chain: batched on its own (see lone_request)
+    bool host;   // a buffer (of a group: of any request) in host memory
 };
+
+// A batch takes requests until the input and output of those in device memory
+// pass this many bytes: the device starts on the first of a burst while the next
+// is planned, and the batches fill each other's tails.  1024 requests of the
+// serving mix at once 2156 -> 1902 us, closed loop 401.7 -> 405.7 GB/s, p99 at 330
+// GB/s 0.51 -> 0.38 ms, p50 and p99 below 180 GB/s unchanged; with four times as
+// much 1929 us.  Requests in host memory do not count: the host link gains
+// nothing (closed loop 131.5 GB/s so, 129.7 where they count).
+constexpr uint64_t kBatchCost = 32ull << 20;
 
 // A CBC-encryption request of more than 512 blocks is one serial chain that
 // a warp walks at about a microsecond per block.  A batch completes as a
 // whole, so requests batched with it would wait for it: it gets a batch of
 // its own instead.
-// A batch takes requests until their input and output pass this many bytes: the
-// device starts on the first of a burst while the next is planned, and the
-// batches fill each other's tails.  1024 requests of the serving mix at once
-// 2156 -> 1902 us, closed loop 401.7 -> 405.7 GB/s, p99 at 330 GB/s 0.51 -> 0.38
-// ms, p50 and p99 below 180 GB/s unchanged; with four times as much 1929 us.
-constexpr uint64_t kBatchCost = 32ull << 20;
 constexpr uint64_t kLoneChainBlocks = 512;
 bool lone_request(const tdes_desc_t& d) {
     return d.mode == TDES_MODE_CBC_ENCRYPT && d.nbytes / 8 > kLoneChainBlocks;
@@ -286,11 +290,13 @@ struct tdes_server {
                 if (queued.load(std::memory_order_acquire) == 0) break;  // nothing to take
                 {
                     std::lock_guard<std::mutex> lock(mu);
-                    while (!queue.empty() && take.size() < cfg.max_batch && cost < kBatchCost &&
+                    uint64_t on_device = 0;
+                    while (!queue.empty() && take.size() < cfg.max_batch && on_device < kBatchCost &&
                            admitted + cost + queue.front().cost <= cfg.budget_bytes) {
                         const bool alone = queue.front().alone;
                         if (alone && !take.empty()) break;  // it starts the next batch
                         cost += queue.front().cost;
+                        if (!queue.front().host) on_device += queue.front().cost;
                         take.push_back(queue.front());
                         queue.pop_front();
                         if (alone) break;
@@ -508,7 +514,9 @@ int tdes_server_submit(tdes_server_t* s, const tdes_desc_t* req, uint64_t* ticke
         return sfail(TDES_EINVAL, "NULL argument");
     if (tdes::validate_desc(*req, s->kt->count) != TDES_OK)
         return sfail(TDES_EINVAL, "invalid request descriptor");
-    if (req->nbytes && (!tdes::gpu_addressable(req->in) || !tdes::gpu_addressable(req->out)))
+    bool host = false;
+    if (req->nbytes &&
+        (!tdes::gpu_addressable(req->in, &host) || !tdes::gpu_addressable(req->out, &host)))
         return sfail(TDES_EINVAL, "request buffers must be device memory or pinned host memory");
     const uint64_t cost = cost_of(*req);
     if (cost > s->cfg.budget_bytes)
@@ -522,7 +530,7 @@ int tdes_server_submit(tdes_server_t* s, const tdes_desc_t* req, uint64_t* ticke
         if (req->nbytes == 0) {
             s->complete(t, TDES_OK, now_ns());
         } else {
-            s->queue.push_back({*req, t, cost, s->wants_stage(*req), lone_request(*req)});
+            s->queue.push_back({*req, t, cost, s->wants_stage(*req), lone_request(*req), host});
             s->queued.store(s->queue.size(), std::memory_order_release);
             s->cv_work.notify_one();
             return TDES_OK;
@@ -553,11 +561,13 @@ int tdes_server_submit_group(tdes_server_t* s, const tdes_desc_t* reqs, uint32_t
                              uint64_t* ticket) {
     if (s == nullptr || ticket == nullptr || (reqs == nullptr && count > 0) || count == 0)
         return sfail(TDES_EINVAL, "NULL argument or empty group");
+    bool host = false;  // any buffer of the group in host memory
     for (uint32_t i = 0; i < count; ++i) {  // the whole group is refused before any is queued
         const tdes_desc_t& r = reqs[i];
         if (tdes::validate_desc(r, s->kt->count) != TDES_OK)
             return sfail(TDES_EINVAL, "invalid request descriptor %u of the group", i);
-        if (r.nbytes && (!tdes::gpu_addressable(r.in) || !tdes::gpu_addressable(r.out)))
+        if (r.nbytes &&
+            (!tdes::gpu_addressable(r.in, &host) || !tdes::gpu_addressable(r.out, &host)))
             return sfail(TDES_EINVAL, "request %u: buffers must be device or pinned host memory", i);
         if (cost_of(r) > s->cfg.budget_bytes)
             return sfail(TDES_EINVAL, "request %u exceeds the admission budget", i);
@@ -573,7 +583,7 @@ int tdes_server_submit_group(tdes_server_t* s, const tdes_desc_t* reqs, uint32_t
                 s->complete(t0 + i, TDES_OK, now_ns());
             else
                 s->queue.push_back({reqs[i], t0 + i, cost_of(reqs[i]), s->wants_stage(reqs[i]),
-                                    lone_request(reqs[i])});
+                                    lone_request(reqs[i]), host});
         }
         s->queued.store(s->queue.size(), std::memory_order_release);
         s->cv_work.notify_one();
