@@ -184,9 +184,10 @@ int make_schedule(tdes::Keys24& keys, int stages, tdes_ks_t** out) {
         if (e == cudaSuccess) e = e2;
         cudaStreamDestroy(s);
     }
-    memset(&keys, 0, sizeof keys);
+    tdes::wipe(&keys, sizeof keys);
     if (e != cudaSuccess) {
         cudaFree(mem);
+        tdes::wipe(ks->host_chunk, sizeof ks->host_chunk);
         delete ks;
         return cuda_fail(e, "key-schedule kernel");
     }
@@ -235,7 +236,7 @@ void tdes_key_free(tdes_ks_t* ks) {
     if (cur != ks->device) cudaSetDevice(ks->device);
     cudaFree(ks->mem);
     if (cur >= 0 && cur != ks->device) cudaSetDevice(cur);
-    memset(ks->host_chunk, 0, sizeof ks->host_chunk);
+    tdes::wipe(ks->host_chunk, sizeof ks->host_chunk);
     delete ks;
 }
 

@@ -3,6 +3,7 @@
 #pragma once
 #include <cstddef>
 #include <cstdint>
+#include <cstring>
 #include <cuda_runtime.h>
 
 // The library's key-schedule object (opaque tdes_ks_t in include/tdes.h).
@@ -12,13 +13,20 @@ struct tdes_ks {
     void* mem;              // one cudaMalloc holding everything below
     uint32_t* tab[2];       // bitsliced round-constant tables: [0] encrypt, [1] decrypt
     uint8_t* chunk[2];      // scalar-path round-key groups: [0] encrypt, [1] decrypt
-    uint8_t host_chunk[2][384];  // host copies of the groups (passed to kernels by value)
+    uint8_t host_chunk[2][384];  // host copies of the groups (kernel parameters); wipe() before freeing
 };
 
 namespace tdes {
 
 // Records the message tdes_last_error() returns on this host thread.
 void set_last_error(const char* msg);
+
+// Clears key material.  The compiler may drop a plain memset of memory that is
+// freed or left next; it has to keep this one.
+inline void wipe(void* p, size_t n) {
+    memset(p, 0, n);
+    asm volatile("" : : "r"(p) : "memory");
+}
 
 // True if the GPU can address `p` with the same pointer: device or managed
 // memory, or page-locked host memory mapped into the device address space

@@ -15,7 +15,6 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
-#include <cstring>
 
 #include "tdes_internal.h"
 #include "tdes_keysched.cuh"
@@ -132,13 +131,18 @@ static cudaError_t lanes_launch(const uint8_t* host_chunks, int mode, uint64_t i
     const uint32_t ctas = (uint32_t)sms * per_sm;
     uint32_t threads = ((nblocks + ctas - 1) / ctas + 31u) / 32u * 32u;
     threads = threads > 512u ? 512u : threads;
-    LaneKeys k;
-    memcpy(k.w, host_chunks, sizeof k.w);
+    // The round keys go to the runtime from where the schedule holds them: an
+    // argument by value would leave copies on the stack.
+    static_assert(sizeof(LaneKeys) == sizeof(tdes_ks::host_chunk[0]), "the schedule's round keys");
+    const uint8_t* src = static_cast<const uint8_t*>(in);
+    uint8_t* dst = static_cast<uint8_t*>(out);
+    void* args[] = {const_cast<uint8_t*>(host_chunks), &mode, &iv, &src, &dst, &nblocks};
     // Not started beside the kernel before: the free places it would take are
     // spread unevenly over the SMs (two calls of 1 MiB 20.5 -> 21.7 us).
-    return launch_kernel(tdes_lanes_kernel<ROUNDS>, (nblocks + threads - 1) / threads, threads,
-                         kLaneTableBytes, s, false, k, mode, iv, static_cast<const uint8_t*>(in),
-                         static_cast<uint8_t*>(out), nblocks);
+    e = cudaLaunchKernel((const void*)tdes_lanes_kernel<ROUNDS>, (nblocks + threads - 1) / threads, threads,
+                         args, kLaneTableBytes, s);
+    if (e != cudaSuccess) cudaGetLastError();  // as launch_kernel
+    return e;
 }
 
 cudaError_t launch_small(SmallKeys keys, int stages, int mode, uint64_t iv, const void* in,
