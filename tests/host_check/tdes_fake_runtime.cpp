@@ -10,6 +10,7 @@
 //   sync      ... or whose stream reports an error
 //   params    a per-lane-table call hands the runtime the schedule's own round
 //             keys as the kernel's parameters (no copy is left on a stack)
+//   copies    a key schedule copies nothing back from the device
 #include <cuda_runtime.h>
 
 #include <cstddef>
@@ -26,6 +27,7 @@ static const uint8_t kSub[2][48][48] = TDES_SUBKEY_INIT;
 static void* g_schedule = nullptr;  // the last tdes_ks allocated, and the state of its
 static int g_cleared = -1;          // round keys when it was freed: 1 all zero, 0 not
 static cudaError_t g_launch = cudaSuccess, g_sync = cudaSuccess;
+static int g_copies_back = 0;
 static const void* g_param0 = nullptr;  // the first parameter of the last kernel launched
 
 // ------------------------------------------------------------- allocation
@@ -78,7 +80,8 @@ cudaError_t cudaMalloc(void** p, size_t n) { *p = calloc(1, n); return cudaSucce
 cudaError_t cudaFree(void* p) { free(p); return cudaSuccess; }
 cudaError_t cudaMallocAsync(void** p, size_t n, cudaStream_t) { return cudaMalloc(p, n); }
 cudaError_t cudaFreeAsync(void* p, cudaStream_t) { return cudaFree(p); }
-cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, enum cudaMemcpyKind, cudaStream_t) {
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, enum cudaMemcpyKind kind, cudaStream_t) {
+    g_copies_back += kind == cudaMemcpyDeviceToHost;
     memcpy(d, s, n);
     return cudaSuccess;
 }
@@ -145,6 +148,7 @@ int main(int argc, char** argv) {
         for (int c = 0; c < TDES_SUBKEY_WORDS; ++c)
             want[dir][c] = tdes_subkey_chunk(&k[0][0], &kSub[dir][c / 8][6 * (c % 8)]);
     if (memcmp(ks->host_chunk, want, sizeof want)) return no("the host's round keys are wrong");
+    if (!strcmp(argv[1], "copies") && g_copies_back) return no("copied from the device");
     if (!strcmp(argv[1], "params")) {
         const size_t n = 8 * 40000;
         void* buf = aligned_alloc(16, n);

@@ -39,3 +39,9 @@ def test_round_keys_are_cleared(exe, case):
     """Round keys in host memory are overwritten before the memory is freed, on
     the error paths too, and a launch leaves no copy of them on a stack."""
     _case(exe, case)
+
+
+def test_key_schedule_copies_nothing_back(exe):
+    """The host's round keys are those of the kernel's recipe, without a copy
+    from the device."""
+    _case(exe, "copies")
