@@ -743,10 +743,12 @@ class Server:
         (ticket, count) of the group."""
         entries = list(entries)
         arr, n = make_descs(entries)
+        # before anything is queued: an entry whose buffers cannot be held is refused
+        held = [b for _, _, _, inp, out, _ in entries for b in (inp, out) if not isinstance(b, int)]
         t = ctypes.c_uint64()
         _check(load().tdes_server_submit_group(self.handle, ctypes.addressof(arr), n,
                                                ctypes.byref(t)))
-        self._hold(t.value, n, [b for e in entries for b in e[3:5] if not isinstance(b, int)])
+        self._hold(t.value, n, held)
         return t.value, n
 
     def poll_group(self, group) -> tuple:
