@@ -34,7 +34,7 @@ def server(monkeypatch):
     s.handle = None  # nothing for close() to destroy
 
 
-@pytest.mark.parametrize("kind", [tuple, list, deque, np.array, "unpacks_only"], ids=str)
+@pytest.mark.parametrize("kind", [tuple, list, deque, iter, np.array, "unpacks_only"], ids=str)
 def test_entry_kinds(server, kind):
     x, y = np.zeros(8, np.uint8), np.zeros(8, np.uint8)
 
@@ -56,9 +56,8 @@ def test_entry_kinds(server, kind):
     assert 7 not in server._keep
 
 
-@pytest.mark.parametrize("bad", [(0, 3, 5, 8, 16), iter((0, 3, 5, 8, 16, 8))], ids=["short", "one_pass"])
+@pytest.mark.parametrize("bad", [(0, 3, 5, 8, 16), deque((0, 3, 5, 8, 16, 8, 9)), 5], ids=str)
 def test_nothing_is_queued_for_an_entry_that_is_refused(server, bad):
-    """Five fields, or fields that can be read once only, cannot be held."""
     with pytest.raises((ValueError, TypeError)):
         server.submit_group([(0, 3, 5, 8, 16, 8), bad])
     assert server.lib.queued == [] and server._keep == {}
