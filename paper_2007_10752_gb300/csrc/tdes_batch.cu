@@ -49,8 +49,12 @@ constexpr uint64_t kMixedMinBlocks = 8 * 1024;
 // would spend its full 1024-block work on them anyway.
 constexpr uint64_t kSplitBlocks = 512;
 // From this many blocks of medium messages their pieces are slices of mixed-key
-// tiles instead: a tile's latency (60 us) then is no longer than the scalar
-// items' time, and the blocks cost a third of the logic operations.
+// tiles instead: a tile's latency (47 to 53 us) then is no longer than the scalar
+// items' time, and the blocks cost a third of the logic operations.  One launch at
+// this line, out of L2, scalar items and tiles: messages of 33 blocks 58.5 and 50.3
+// us, of 48 53.4 and 53.9, of 64 52.4 and 51.4, of 512 52.4 and 47.2; eight times as
+// many blocks 335 and 90, 307 and 93, 280 and 67, 280 and 59.  (Before a tile's loads
+// were taken off one another, the tiles lost by up to a fifth at the line.)
 // 4096 records of 64 B to 4 KiB through a context 909 -> 861 us, the 4096-message
 // batch 3482 -> 3461 us, the server's closed loop 391 -> 402 GB/s.
 constexpr uint64_t kMixedSplitBlocks = 128 * 1024;
@@ -353,21 +357,41 @@ __device__ __forceinline__ void batch_mixed_tile(const BatchParams& p, uint32_t 
     uint32_t* wtab = reinterpret_cast<uint32_t*>(g_dyn + (size_t)warp * kWarpSmemBytes);
     const MSlice* sl = p.m_slices + 32ull * tile;
     {
+        // Four words a load, the next four under way while these are transposed: a
+        // word at a time, each behind the one before, the loads took a third of a
+        // lone tile's 45 us.
         const uint32_t kd = sl[lane].keydir;
-        const uint32_t* row = p.keypacked + ((uint64_t)(kd >> 1) * 2 + (kd & 1u)) * kPackedWords;
+        const uint4* row = reinterpret_cast<const uint4*>(
+            p.keypacked + ((uint64_t)(kd >> 1) * 2 + (kd & 1u)) * kPackedWords);
+        static_assert(kPackedWords % 4 == 0, "rows of 16-byte words");
         __syncwarp();
+        uint4 w = __ldg(row);
 #pragma unroll 1
-        for (int q = 0; q < kPackedWords; ++q)
-            wtab[32 * q + lane] = transpose_lanes32(__ldg(row + q), lane);
+        for (int q = 0; q < kPackedWords / 4; ++q) {
+            const uint4 next = __ldg(row + min(q + 1, kPackedWords / 4 - 1));
+            uint32_t* t = wtab + 128 * q + lane;
+            t[0] = transpose_lanes32(w.x, lane);
+            t[32] = transpose_lanes32(w.y, lane);
+            t[64] = transpose_lanes32(w.z, lane);
+            t[96] = transpose_lanes32(w.w, lane);
+            w = next;
+        }
         __syncwarp();
     }
     uint32_t A0[32], A1[32];
+    // lane s holds slice s's record, so that a slice's message and data are not
+    // loaded behind it, once for the blocks and once for what follows the rounds
+    MSlice mine = sl[lane];
+    auto slice = [&](int s) {
+        return MSlice{__shfl_sync(0xFFFFFFFFu, mine.msg0, s), __shfl_sync(0xFFFFFFFFu, mine.starts, s),
+                      __shfl_sync(0xFFFFFFFFu, mine.nvalid, s), 0u};
+    };
 #pragma unroll
     for (int s = 0; s < 32; ++s) {
         uint32_t mi, b;
         A0[s] = 0u;
         A1[s] = 0u;
-        if (mixed_slot(p, sl[s], lane, &mi, &b)) {
+        if (mixed_slot(p, slice(s), lane, &mi, &b)) {
             const BatchMsg m = p.msgs[mi];
             if (m.mode == TDES_MODE_CTR) {
                 A0[s] = bswap32d((uint32_t)(m.iv >> 32));
@@ -380,10 +404,11 @@ __device__ __forceinline__ void batch_mixed_tile(const BatchParams& p, uint32_t 
         }
     }
     tdes_process32_mixed(A0, A1, wtab);
+    mine = sl[lane];  // not kept in registers through the rounds
 #pragma unroll
     for (int s = 0; s < 32; ++s) {
         uint32_t mi, b;
-        const bool ok = mixed_slot(p, sl[s], lane, &mi, &b);
+        const bool ok = mixed_slot(p, slice(s), lane, &mi, &b);
         BatchMsg m;
         if (ok) {
             m = p.msgs[mi];

@@ -1,0 +1,55 @@
+"""Where a rule takes a call to another path, the call takes no longer there than
+its neighbour on the other side.  Both are timed in turn, so that whatever else
+moves moves both; the limits leave 8% for the events' grain (2 us) and spread."""
+import numpy as np
+import pytest
+
+from paper_2007_10752_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _ratio(a, b, rows=1, rounds=60):
+    """Time of `rows` calls of a, out of L2, over that of b, taken in turn (means
+    of the middle half)."""
+    flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
+    times = ([], [])
+    for i in range(rounds + 3):
+        for call, out in zip((a, b), times):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            flush.zero_()
+            e0.record()
+            for _ in range(rows):
+                call()
+            e1.record()
+            e1.synchronize()
+            if i >= 3:
+                out.append(e0.elapsed_time(e1))
+    mid = [np.mean(sorted(t)[rounds // 4:-(rounds // 4)]) for t in times]
+    return float(mid[0] / mid[1])
+
+
+def _medium(cuda_lib, nb, blocks):
+    """A plan of messages of nb blocks, `blocks` in all or the last ones fewer."""
+    n = blocks // nb
+    src = torch.zeros(8 * nb * n, dtype=torch.uint8, device="cuda")
+    synth.fill_device(src, nb)
+    dst = torch.empty_like(src)
+    kt = cuda_lib.KeyTable(synth.key_triples(nb, 64))
+    plan = cuda_lib.Batch(kt, [((0, 2, 3, 1)[i % 4], i % 64, i << 32, src.data_ptr() + 8 * nb * i,
+                                dst.data_ptr() + 8 * nb * i, 8 * nb) for i in range(n)])
+    return plan, (kt, src, dst)
+
+
+@pytest.mark.parametrize("nb", [33, 48, 64, 512])
+def test_medium_messages_past_the_line(cuda_lib, nb):
+    """131072 blocks of medium messages as mixed-key tiles, and one message fewer
+    as scalar items."""
+    blocks = -(-131072 // nb) * nb
+    past, hold = _medium(cuda_lib, nb, blocks)
+    before, hold2 = _medium(cuda_lib, nb, blocks - nb)
+    assert past.info()["n_mixed_tiles"] > 0 and before.info()["n_mixed_tiles"] == 0
+    r = _ratio(past.launch_graph, before.launch_graph)
+    del hold, hold2
+    assert r <= 1.08, r
