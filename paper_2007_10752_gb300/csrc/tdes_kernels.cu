@@ -133,9 +133,8 @@ __device__ __forceinline__ uint32_t bswap32(uint32_t x) { return __byte_perm(x, 
 // the other, so that a last pass with fewer tiles than warps loads every
 // sub-partition alike: a tile alone on one takes 17 us, four together 44 us.
 // (Consecutive tiles per CTA put the 84 last tiles of 1300 on 11 SMs: 50.6
-// against 35.4 us.  In a kernel that starts beside the one before, slots are
-// taken as they come free, and 700 tiles take 30 instead of 27 us.)  %warpid is only a hint: any values give each warp a rank
-// of its own.  publish_slot before a barrier, first_tile after it.
+// against 35.4 us.)  %warpid is only a hint: any values give each warp a rank of
+// its own.  publish_slot before a barrier, first_tile after it.
 __device__ __forceinline__ void publish_slot(uint32_t* slots) {
     uint32_t slot;
     asm("mov.u32 %0, %%warpid;" : "=r"(slot));
@@ -163,14 +162,13 @@ template <int MODE>
 __device__ __noinline__ void scalar_tail(Tail tail, uint64_t first, uint64_t iv, const uint8_t* in,
                                          uint8_t* out, uint32_t* __restrict__ keys,
                                          uint8_t* __restrict__ tab) {
-    const uint32_t share = ((tail.n + gridDim.x - 1) / gridDim.x + 31u) / 32u * 32u;
-    const uint32_t b0 = blockIdx.x * share;
+    const uint32_t b0 = blockIdx.x * tail.share;
     if (b0 >= tail.n) return;
     __syncthreads();  // every warp has left its tile buffer and the round constants
     lane_tables(tab, &kTailSP[0][0]);
     if (threadIdx.x < TDES_SUBKEY_WORDS / 4) keys[threadIdx.x] = __ldg(tail.keys + threadIdx.x);
     __syncthreads();
-    const uint32_t end = min(b0 + share, tail.n), lane4 = (threadIdx.x & 31u) * 4u;
+    const uint32_t end = min(b0 + tail.share, tail.n), lane4 = (threadIdx.x & 31u) * 4u;
     const uint64_t* p = reinterpret_cast<const uint64_t*>(in) + first;
     uint64_t* q = reinterpret_cast<uint64_t*>(out) + first;
     for (uint32_t b = b0 + threadIdx.x; b < end; b += blockDim.x) {
@@ -302,13 +300,25 @@ static cudaError_t ensure_dyn_smem() {
 // step there costs a lone tile's 17 us), else up to 128 (7 us).
 static uint64_t tail_split(int stages, bool vec16, Geometry g, const uint8_t* chunks,
                            uint64_t nblocks, Tail* tail) {
-    *tail = Tail{nullptr, 0};
+    *tail = Tail{nullptr, 0, 0};
     if (stages != 3 || !vec16 || chunks == nullptr || g.threads != 32 * kWideWarps) return nblocks;
     const uint64_t step = 4ull * g.sms * kTileBlocks, steps = nblocks / step;
     const uint64_t rest = nblocks - steps * step;
     if (steps == 0 || rest > (steps % 4 == 0 ? 320u : 128u) * (uint64_t)kTileBlocks) return nblocks;
     tail->keys = reinterpret_cast<const uint32_t*>(chunks);
     tail->n = (uint32_t)rest;
+    // Whole warps, the same in every CTA that has a share.  With one step of tiles
+    // a CTA ends as soon as its share does, and the call after it starts in its
+    // place (launch_kernel): five, six, nine or more warps that load the
+    // sub-partitions unevenly then delay that call's tiles, and are made a multiple
+    // of four on fewer CTAs.  ECB calls in a row: 608 + 41 tiles 28.8 -> 22.4 us, + 77
+    // 31.5 -> 24.6, + 91 31.4 -> 24.6, + 128 32.3 -> 26.1 (up to 28 where their CTAs
+    // find other places; all-tile calls, + 160, 25.8); 7 warps are as good as 8, in CBC
+    // decryption better (+ 66 21.9 and 23.4).  After more steps it gains nothing
+    // (1216 + 66 32.1 and 32.7).
+    uint32_t warps = ((uint32_t)rest + 32u * g.grid - 1) / (32u * g.grid);
+    if (steps == 1 && warps > 4 && warps != 7) warps = (warps + 3) / 4 * 4;
+    tail->share = 32 * warps;
     return steps * step;
 }
 
