@@ -92,12 +92,11 @@ struct Geometry {
 };
 
 // The blocks of a call that run one per thread after the kernel's tiles: n of
-// them, right after the tiles' blocks, share to a CTA; keys is the call's scalar
-// round-key groups on the device.
+// them, right after the tiles' blocks; keys is the call's scalar round-key
+// groups on the device.
 struct Tail {
     const uint32_t* keys;
     uint32_t n;
-    uint32_t share;
 };
 Geometry geometry_for(uint64_t ntiles, int kernel_id, int device);
 

@@ -128,28 +128,46 @@ __device__ __forceinline__ uint32_t bswap32(uint32_t x) { return __byte_perm(x, 
 
 // ------------------------------------------------ first tile of a warp, tail
 // Tile of a warp's first pass (the later ones follow a stride of all warps).
-// The passes run CTA by CTA within a rank, and a CTA ranks its warps by SM
-// sub-partition, from 0 in the CTA that holds the SM's warp slot 0 and from 2 in
-// the other, so that a last pass with fewer tiles than warps loads every
-// sub-partition alike: a tile alone on one takes 17 us, four together 44 us.
-// (Consecutive tiles per CTA put the 84 last tiles of 1300 on 11 SMs: 50.6
-// against 35.4 us.)  %warpid is only a hint: any values give each warp a rank of
-// its own.  publish_slot before a barrier, first_tile after it.
+// The passes run CTA by CTA within a rank, and a CTA ranks its warps so that every
+// four ranks are one warp of each SM sub-partition, from sub-partition 0 in the CTA
+// that holds the SM's warp slot 0 and from 2 in the other: a last pass with fewer
+// tiles than warps then loads every sub-partition alike (a tile alone on one takes
+// 17 us, four together 44 us).  A warp slot's sub-partition is its low two bits.
+// Consecutive tiles per CTA put the 84 last tiles of 1300 on 11 SMs: 50.6 against
+// 35.4 us.  Ranks in the order of the slots did the same in a CTA whose slots are
+// not consecutive, as a kernel that starts beside the one before gets them (0, 1, 3,
+// 4, 5, 6, 7, 10: two of the first four ranks on sub-partition 0): calls of 1100
+// tiles with one of 300 before each 57.6 -> 45.4 us, of 700 69.7 -> 50.1, in a row
+// 25.9 -> 25.6, and calls of 608 + 91 tiles in a row 31.4 -> 24.6.
+// %warpid is only a hint: any slots give each warp a rank of its own.
+// publish_slot before a barrier, first_tile after it.
 __device__ __forceinline__ void publish_slot(uint32_t* slots) {
     uint32_t slot;
     asm("mov.u32 %0, %%warpid;" : "=r"(slot));
     if ((threadIdx.x & 31u) == 0) slots[threadIdx.x >> 5] = slot;
 }
-__device__ __forceinline__ uint32_t first_tile(const uint32_t* slots) {
-    const uint32_t warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
-    uint32_t lowest = slots[0];
-    for (uint32_t w = 1; w < warps; ++w) lowest = min(lowest, slots[w]);
-    const uint32_t turn = lowest ? 2u : 0u;
-    const uint32_t mine = (slots[warp] ^ turn) * kWideWarps + warp;
-    uint32_t rank = 0;
-    for (uint32_t w = 0; w < warps; ++w) rank += (slots[w] ^ turn) * kWideWarps + w < mine;
-    return rank * gridDim.x + blockIdx.x;
+__device__ __forceinline__ uint32_t first_tile_inline(const uint32_t* slots) {
+    if (blockDim.x == 32) return blockIdx.x;  // else kWideWarps warps
+    static_assert(kWideWarps == 8, "two warps of a CTA on each of four sub-partitions");
+    const uint32_t me = threadIdx.x % kWideWarps;  // a warp's lanes w, w + 8, ... rank warp w
+    const uint32_t slot = slots[me];
+    uint32_t lowest = slot, earlier = 0;
+#pragma unroll
+    for (int w = 0; w < kWideWarps; ++w) {
+        const uint32_t s = slots[w];
+        lowest = min(lowest, s);
+        earlier += ((s ^ slot) & 3u) == 0 && s < slot;  // before it on its sub-partition
+    }
+    uint32_t rank = 4u * earlier + ((slot ^ (lowest ? 2u : 0u)) & 3u);
+    // eight different ranks below eight, or else the warps' own order
+    if (__reduce_or_sync(0xFFFFFFFFu, 1u << rank) != (1u << kWideWarps) - 1u) rank = me;
+    return __shfl_sync(0xFFFFFFFFu, rank, threadIdx.x >> 5) * gridDim.x + blockIdx.x;
 }
+
+// A real call: inlined, it cost the 8-byte-aligned CTR and CBC kernels a spilled
+// register and 1 GiB ECB 11 us (2451 and 2440); the 16-byte-aligned CBC kernel
+// takes it inlined (200 MB 476.4 us, with the call 478.7).
+__device__ __noinline__ uint32_t first_tile(const uint32_t* slots) { return first_tile_inline(slots); }
 
 // The blocks after the last whole round of tiles (tail_split): one block per
 // thread in every CTA, on the per-lane tables of tdes_lanes.cuh in the place
@@ -162,13 +180,14 @@ template <int MODE>
 __device__ __noinline__ void scalar_tail(Tail tail, uint64_t first, uint64_t iv, const uint8_t* in,
                                          uint8_t* out, uint32_t* __restrict__ keys,
                                          uint8_t* __restrict__ tab) {
-    const uint32_t b0 = blockIdx.x * tail.share;
+    const uint32_t share = ((tail.n + gridDim.x - 1) / gridDim.x + 31u) / 32u * 32u;
+    const uint32_t b0 = blockIdx.x * share;
     if (b0 >= tail.n) return;
     __syncthreads();  // every warp has left its tile buffer and the round constants
     lane_tables(tab, &kTailSP[0][0]);
     if (threadIdx.x < TDES_SUBKEY_WORDS / 4) keys[threadIdx.x] = __ldg(tail.keys + threadIdx.x);
     __syncthreads();
-    const uint32_t end = min(b0 + tail.share, tail.n), lane4 = (threadIdx.x & 31u) * 4u;
+    const uint32_t end = min(b0 + share, tail.n), lane4 = (threadIdx.x & 31u) * 4u;
     const uint64_t* p = reinterpret_cast<const uint64_t*>(in) + first;
     uint64_t* q = reinterpret_cast<uint64_t*>(out) + first;
     for (uint32_t b = b0 + threadIdx.x; b < end; b += blockDim.x) {
@@ -210,6 +229,7 @@ tdes_ecb_kernel(const uint32_t* __restrict__ table, const uint8_t* in, uint8_t* 
     stage_table<STAGES>(tab, table);
     publish_slot(slots);
     __syncthreads();
+    const uint32_t first = first_tile(slots);
     wait_for_primary();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warps = blockDim.x >> 5;
@@ -218,7 +238,7 @@ tdes_ecb_kernel(const uint32_t* __restrict__ table, const uint8_t* in, uint8_t* 
     const uint32_t ntiles = (uint32_t)((nblocks + kTileBlocks - 1) / kTileBlocks);
     const uint32_t nfull = (uint32_t)(nblocks / kTileBlocks);  // tiles [0, nfull) are full
     const uint32_t stride = gridDim.x * warps;
-    uint32_t t = first_tile(slots);
+    uint32_t t = first;
     if (VEC && t < nfull) {
         const uint4* p = reinterpret_cast<const uint4*>(in) + (uint64_t)t * (kTileBlocks / 2) + lane;
 #pragma unroll
@@ -300,25 +320,13 @@ static cudaError_t ensure_dyn_smem() {
 // step there costs a lone tile's 17 us), else up to 128 (7 us).
 static uint64_t tail_split(int stages, bool vec16, Geometry g, const uint8_t* chunks,
                            uint64_t nblocks, Tail* tail) {
-    *tail = Tail{nullptr, 0, 0};
+    *tail = Tail{nullptr, 0};
     if (stages != 3 || !vec16 || chunks == nullptr || g.threads != 32 * kWideWarps) return nblocks;
     const uint64_t step = 4ull * g.sms * kTileBlocks, steps = nblocks / step;
     const uint64_t rest = nblocks - steps * step;
     if (steps == 0 || rest > (steps % 4 == 0 ? 320u : 128u) * (uint64_t)kTileBlocks) return nblocks;
     tail->keys = reinterpret_cast<const uint32_t*>(chunks);
     tail->n = (uint32_t)rest;
-    // Whole warps, the same in every CTA that has a share.  With one step of tiles
-    // a CTA ends as soon as its share does, and the call after it starts in its
-    // place (launch_kernel): five, six, nine or more warps that load the
-    // sub-partitions unevenly then delay that call's tiles, and are made a multiple
-    // of four on fewer CTAs.  ECB calls in a row: 608 + 41 tiles 28.8 -> 22.4 us, + 77
-    // 31.5 -> 24.6, + 91 31.4 -> 24.6, + 128 32.3 -> 26.1 (up to 28 where their CTAs
-    // find other places; all-tile calls, + 160, 25.8); 7 warps are as good as 8, in CBC
-    // decryption better (+ 66 21.9 and 23.4).  After more steps it gains nothing
-    // (1216 + 66 32.1 and 32.7).
-    uint32_t warps = ((uint32_t)rest + 32u * g.grid - 1) / (32u * g.grid);
-    if (steps == 1 && warps > 4 && warps != 7) warps = (warps + 3) / 4 * 4;
-    tail->share = 32 * warps;
     return steps * step;
 }
 
@@ -357,6 +365,7 @@ tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr
     stage_table<STAGES>(tab, table);
     publish_slot(slots);
     __syncthreads();
+    const uint32_t first = first_tile(slots);
     wait_for_primary();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warps = blockDim.x >> 5;
@@ -367,7 +376,7 @@ tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr
     // Tile indices fit 32 bits: the host caps a call below 2^31 tiles.
     using Idx = typename std::conditional<VEC, uint64_t, uint32_t>::type;
     const Idx ntiles = (Idx)((nblocks + kTileBlocks - 1) / kTileBlocks);
-    for (Idx t = first_tile(slots); t < ntiles; t += (Idx)gridDim.x * warps) {
+    for (Idx t = first; t < ntiles; t += (Idx)gridDim.x * warps) {
         const uint64_t b0 = (uint64_t)t * kTileBlocks;
         const bool full = VEC && b0 + kTileBlocks <= nblocks;
         if (full) {  // each lane copies, and later reads back, only its own 16 x 16 bytes
@@ -491,6 +500,7 @@ tdes_cbc_dec_kernel(const uint32_t* __restrict__ table, uint64_t iv, const uint8
     stage_table<STAGES>(tab, table);
     publish_slot(slots);
     __syncthreads();
+    const uint32_t first = VEC ? first_tile_inline(slots) : first_tile(slots);
     wait_for_primary();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warps = blockDim.x >> 5;
@@ -501,7 +511,7 @@ tdes_cbc_dec_kernel(const uint32_t* __restrict__ table, uint64_t iv, const uint8
     const uint32_t stride = gridDim.x * warps;
     const uint2 ivw = make_uint2(bswap32((uint32_t)(iv >> 32)), bswap32((uint32_t)iv));
     const uint2* c = reinterpret_cast<const uint2*>(in);
-    uint32_t t = first_tile(slots);
+    uint32_t t = first;
     if (VEC && t < nfull) {  // full tiles are prefetched one ahead, as in ECB
         const uint4* p = reinterpret_cast<const uint4*>(in) + (uint64_t)t * (kTileBlocks / 2) + lane;
 #pragma unroll

@@ -55,24 +55,46 @@ def test_medium_messages_past_the_line(cuda_lib, nb):
     assert r <= 1.08, r
 
 
-@pytest.mark.parametrize("mode", ["ecb", "ctr", "cbc_dec"])
-@pytest.mark.parametrize("tail", [81, 120, 128])
-def test_tails_in_a_row(cuda_lib, mode, tail):
-    """Calls of one step of tiles (608) and a tail, one after another, take no
-    longer than calls of 32 tiles more than the longest tail, all of them whole
-    tiles.  15%: the calls' CTAs find their places one way or another."""
-    step = 4 * torch.cuda.get_device_properties(0).multi_processor_count
-    ks = cuda_lib.KeySchedule.from_triple(synth.key_triple(step))
-    x = torch.zeros(8192 * (step + 160), dtype=torch.uint8, device="cuda")
+def _single_key(cuda_lib, mode, longest):
+    """A function that makes the call of a number of tiles."""
+    ks = cuda_lib.KeySchedule.from_triple(synth.key_triple(longest))
+    x = torch.zeros(8192 * longest, dtype=torch.uint8, device="cuda")
     y = torch.empty_like(x)
 
     def call(tiles):
-        a, b = x[:8192 * (step + tiles)], y[:8192 * (step + tiles)]
+        a, b = x[:int(8192 * tiles)], y[:int(8192 * tiles)]
         if mode == "ecb":
             return lambda: cuda_lib.tdes_ecb_encrypt(ks, a, b)
         if mode == "ctr":
             return lambda: cuda_lib.tdes_ctr_crypt(ks, 5, 0, a, b)
         return lambda: cuda_lib.tdes_cbc_decrypt(ks, 9, a, b)
 
-    r = _ratio(call(tail), call(160), rows=50, rounds=20)
-    assert r <= 1.15, r
+    return call
+
+
+@pytest.mark.parametrize("mode", ["ecb", "ctr", "cbc_dec"])
+@pytest.mark.parametrize("tail", [81, 120, 128])
+def test_tails_in_a_row(cuda_lib, mode, tail):
+    """Calls of one step of tiles (608) and a tail, one after another, take no
+    longer than calls of 32 tiles more than the longest tail, all of them whole
+    tiles."""
+    step = 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    call = _single_key(cuda_lib, mode, step + 160)
+    r = _ratio(call(step + tail), call(step + 160), rows=50, rounds=20)
+    assert r <= 1.08, r
+
+
+@pytest.mark.parametrize("mode", ["ecb", "ctr", "cbc_dec"])
+@pytest.mark.parametrize("before,more", [(300, 608), (700, 800)], ids=str)
+def test_calls_after_uneven_ones(cuda_lib, mode, before, more):
+    """A wide call that starts beside a call which loads the SMs unevenly: the two
+    take no longer than with a larger, even call in its place."""
+    call = _single_key(cuda_lib, mode, 1100)
+    wide = call(1100)
+
+    def pair(tiles):
+        first = call(tiles)
+        return lambda: (first(), wide())
+
+    r = _ratio(pair(before), pair(more), rows=20, rounds=20)
+    assert r <= 1.08, r

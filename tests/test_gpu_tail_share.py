@@ -1,6 +1,5 @@
-"""Tails after one step of tiles whose share of a CTA is rounded up to whole
-rounds of four warps, so that not every CTA has one: every block against the
-oracle, just around the sizes where the rounding changes."""
+"""Tails after one step of tiles around the numbers of blocks at which a CTA's
+share takes one more warp, whole and ragged: every block against the oracle."""
 import os
 
 import numpy as np
@@ -14,12 +13,11 @@ pytestmark = pytest.mark.gpu
 NCPU = max(1, min(16, os.cpu_count() or 1))
 
 
-# extra blocks for each CTA (two on each SM): the last and first of a number of
-# warps, with the CTAs' shares whole and ragged
+# blocks for each CTA (two on each SM), and a few more or fewer in all
 @pytest.mark.parametrize("mode", ["ecb_enc", "ecb_dec", "ctr", "cbc_dec"])
 @pytest.mark.parametrize("per_cta,more", [(128, 0), (128, 1), (160, 3), (192, 1), (224, 0), (224, 1), (300, 77),
                                           (384, 1), (431, -5)], ids=str)
-def test_rounded_shares(cuda_lib, per_cta, more, mode):
+def test_shares(cuda_lib, per_cta, more, mode):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     n = 4 * sms * 1024 + 2 * sms * per_cta + more
     keys, iv, nonce, ctr0 = synth.key_triple(n), synth.iv64(n), synth.nonce32(n), 2**32 - n
