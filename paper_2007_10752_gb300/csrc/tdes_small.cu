@@ -73,8 +73,14 @@ tdes_small_kernel(const uint8_t* __restrict__ chunks, int mode, uint64_t iv, con
 // ---- one block per thread, a copy of the tables per lane (tdes_lanes.cuh) ----
 constexpr uint64_t kLanesMinBlocks = 28672;
 // Calls of so few CTAs of tdes_small_kernel may start beside the kernel before
-// (launch_kernel): wherever they find a place, an SM has room for all of them.
+// (launch_kernel).  Where that one fills the GPU they find their places as its
+// first CTAs end, and all 16 together on one SM took 13 us instead of 3.5: two or more
+// ask for so much shared memory (of which they use 2.4 KB) that an SM has room for
+// three or four (1100 tiles after 2048 blocks, again and again: 55 us, 30.4 so; both
+// waiting for the call before 39.3).  With 64 or 100 KB each 29.3, but then none runs
+// beside a batch kernel's three CTAs of four warps on an SM (0.1 -> 3.2 ms).
 constexpr uint64_t kOverlapCtas = 16;
+constexpr size_t kOverlapSmem = 48 * 1024;
 
 template <int ROUNDS>
 __global__ void __launch_bounds__(512, 3)
@@ -152,8 +158,10 @@ cudaError_t launch_small(SmallKeys keys, int stages, int mode, uint64_t iv, cons
                    ? lanes_launch<16>(keys.host, mode, iv, in, out, (uint32_t)nblocks, s)
                    : lanes_launch<48>(keys.host, mode, iv, in, out, (uint32_t)nblocks, s);
     const uint64_t grid = (nblocks + threads - 1) / threads;
+    const bool overlap = grid <= kOverlapCtas;
+    const size_t smem = overlap && grid > 1 ? kOverlapSmem - sizeof(SmallTables) : 0;
     return launch_kernel(stages == 1 ? tdes_small_kernel<16> : tdes_small_kernel<48>,
-                         (unsigned)grid, (unsigned)threads, 0, s, grid <= kOverlapCtas, keys.dev, mode, iv,
+                         (unsigned)grid, (unsigned)threads, smem, s, overlap, keys.dev, mode, iv,
                          static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out), nblocks);
 }
 

@@ -98,3 +98,13 @@ def test_calls_after_uneven_ones(cuda_lib, mode, before, more):
 
     r = _ratio(pair(before), pair(more), rows=20, rounds=20)
     assert r <= 1.08, r
+
+
+def test_small_calls_between_wide_ones(cuda_lib):
+    """A call of 2048 blocks, 16 CTAs, that starts as a wide call's CTAs end: the two
+    take little longer than with a call of one CTA (alone the larger takes 0.4 us
+    longer)."""
+    call = _single_key(cuda_lib, "ecb", 1100)
+    wide, many, one = call(1100), call(2), call(1 / 16)
+    r = _ratio(lambda: (many(), wide()), lambda: (one(), wide()), rows=20, rounds=20)
+    assert r <= 1.15, r
