@@ -87,7 +87,6 @@ bool aligned16(const void* in, const void* out) {
 
 // Calls of at most this many blocks run one block per thread (tdes_small.cu).
 std::atomic<uint64_t> g_small_cutoff{TDES_SMALL_CUTOFF_DEFAULT};
-constexpr int kSmallThreads = 128;  // per CTA: spreads a small call over many SMs
 
 }  // namespace
 
@@ -263,7 +262,7 @@ static int ecb(const tdes_ks_t* ks, int dir, const void* in, void* out, size_t n
     cudaError_t e;
     if (nblocks <= g_small_cutoff.load(std::memory_order_relaxed)) {
         e = tdes::launch_small(tdes::small_keys(ks, dir), ks->stages, tdes::kSmallEcb, 0, in, out, nblocks,
-                               kSmallThreads, s);
+                               tdes::kSmallThreads, s);
     } else {
         const uint64_t ntiles = (nblocks + tdes::kTileBlocks - 1) / tdes::kTileBlocks;
         const tdes::Geometry g = tdes::geometry_for(ntiles, tdes::kEcb, ks->device);
@@ -294,7 +293,7 @@ int tdes_ctr_crypt(const tdes_ks_t* ks, uint32_t nonce, uint32_t ctr0, const voi
     cudaError_t e;
     if (nblocks <= g_small_cutoff.load(std::memory_order_relaxed)) {
         e = tdes::launch_small(tdes::small_keys(ks, 0), ks->stages, tdes::kSmallCtr,
-                               (uint64_t)nonce << 32 | ctr0, in, out, nblocks, kSmallThreads, s);
+                               (uint64_t)nonce << 32 | ctr0, in, out, nblocks, tdes::kSmallThreads, s);
     } else {
         const uint64_t ntiles = (nblocks + tdes::kTileBlocks - 1) / tdes::kTileBlocks;
         const tdes::Geometry g = tdes::geometry_for(ntiles, tdes::kCtr, ks->device);
@@ -312,7 +311,7 @@ int tdes_cbc_decrypt(const tdes_ks_t* ks, uint64_t iv, const void* in, void* out
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     // one block per thread; in place only as a single CTA (all reads before writes)
     if (nblocks <= g_small_cutoff.load(std::memory_order_relaxed) && (in != out || nblocks <= 1024)) {
-        const int threads = in != out ? kSmallThreads : (int)((nblocks + 31) / 32 * 32);
+        const int threads = in != out ? tdes::kSmallThreads : (int)((nblocks + 31) / 32 * 32);
         cudaError_t e = tdes::launch_small(tdes::small_keys(ks, 1), ks->stages, tdes::kSmallCbcDec, iv, in,
                                            out, nblocks, threads, s);
         return e == cudaSuccess ? TDES_OK : cuda_fail(e, "CBC-decrypt kernel launch");

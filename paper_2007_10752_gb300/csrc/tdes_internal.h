@@ -122,6 +122,7 @@ cudaError_t launch_cbc_enc(const uint8_t* chunk_enc, int stages, uint64_t iv, co
 // One block per thread (tdes_small.cu), for calls too small to fill the GPU
 // with bitsliced tiles.  keys: the call's scalar round-key groups of the
 // wanted direction, on the device and on the host; iv: the CBC IV, or nonce << 32 | ctr0 for CTR.
+constexpr int kSmallThreads = 128;  // per CTA: spreads a small call over many SMs
 enum SmallMode { kSmallEcb = 0, kSmallCtr = 1, kSmallCbcDec = 2 };
 struct SmallKeys {
     const uint8_t* dev;

@@ -40,7 +40,8 @@ __device__ __forceinline__ uint64_t small_load_be(const uint8_t* p, uint64_t i) 
 // (each thread reads and writes only its own block); for CBC decryption the
 // host uses this kernel in place only with a single CTA, whose threads all
 // read before any writes.
-template <int ROUNDS>
+// SPREAD: only the first kSmallThreads threads of a CTA take a block (launch_small).
+template <int ROUNDS, bool SPREAD>
 __global__ void __launch_bounds__(1024)
 tdes_small_kernel(const uint8_t* __restrict__ chunks, int mode, uint64_t iv, const uint8_t* in,
                   uint8_t* out, uint64_t nblocks) {
@@ -51,7 +52,9 @@ tdes_small_kernel(const uint8_t* __restrict__ chunks, int mode, uint64_t iv, con
     for (int i = threadIdx.x; i < TDES_SUBKEY_WORDS / 4; i += blockDim.x)
         st.keys[i] = __ldg(reinterpret_cast<const uint32_t*>(chunks) + i);
     wait_for_primary();
-    const uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (SPREAD)
+        b = threadIdx.x < kSmallThreads ? (uint64_t)blockIdx.x * kSmallThreads + threadIdx.x : nblocks;
     uint64_t x = 0, prev = 0;
     if (b < nblocks) {
         if (mode == kSmallCtr) {
@@ -74,13 +77,14 @@ tdes_small_kernel(const uint8_t* __restrict__ chunks, int mode, uint64_t iv, con
 constexpr uint64_t kLanesMinBlocks = 28672;
 // Calls of so few CTAs of tdes_small_kernel may start beside the kernel before
 // (launch_kernel).  Where that one fills the GPU they find their places as its
-// first CTAs end, and all 16 together on one SM took 13 us instead of 3.5: two or more
-// ask for so much shared memory (of which they use 2.4 KB) that an SM has room for
-// three or four (1100 tiles after 2048 blocks, again and again: 55 us, 30.4 so; both
-// waiting for the call before 39.3).  With 64 or 100 KB each 29.3, but then none runs
-// beside a batch kernel's three CTAs of four warps on an SM (0.1 -> 3.2 ms).
+// first CTAs end, and all 16 together on one SM took 13 us instead of 3.5.  Two or more
+// therefore get 512 threads, of which those past the CTA's blocks only help to stage
+// the table, so that an SM has room for two to four: 1100 tiles after 2048 blocks,
+// again and again, 55 -> 31.9 us (both waiting for the call before: 39.3; with 256
+// threads 36.5).  Shared memory asked for instead did the same, but a CTA of 48 KB
+// waits for an idle SM, beside a 1 GiB call for that call's end.
 constexpr uint64_t kOverlapCtas = 16;
-constexpr size_t kOverlapSmem = 48 * 1024;
+constexpr int kOverlapThreads = 512;
 
 template <int ROUNDS>
 __global__ void __launch_bounds__(512, 3)
@@ -158,11 +162,15 @@ cudaError_t launch_small(SmallKeys keys, int stages, int mode, uint64_t iv, cons
                    ? lanes_launch<16>(keys.host, mode, iv, in, out, (uint32_t)nblocks, s)
                    : lanes_launch<48>(keys.host, mode, iv, in, out, (uint32_t)nblocks, s);
     const uint64_t grid = (nblocks + threads - 1) / threads;
-    const bool overlap = grid <= kOverlapCtas;
-    const size_t smem = overlap && grid > 1 ? kOverlapSmem - sizeof(SmallTables) : 0;
-    return launch_kernel(stages == 1 ? tdes_small_kernel<16> : tdes_small_kernel<48>,
-                         (unsigned)grid, (unsigned)threads, smem, s, overlap, keys.dev, mode, iv,
-                         static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out), nblocks);
+    auto launch = [&](auto kernel, unsigned cta) {
+        return launch_kernel(kernel, (unsigned)grid, cta, 0, s, grid <= kOverlapCtas, keys.dev, mode, iv,
+                             static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out), nblocks);
+    };
+    if (threads == kSmallThreads && grid > 1 && grid <= kOverlapCtas)
+        return launch(stages == 1 ? tdes_small_kernel<16, true> : tdes_small_kernel<48, true>,
+                      kOverlapThreads);
+    return launch(stages == 1 ? tdes_small_kernel<16, false> : tdes_small_kernel<48, false>,
+                  (unsigned)threads);
 }
 
 }  // namespace tdes
