@@ -133,7 +133,7 @@ Geometry geometry_for(uint64_t ntiles, int kernel_id, int device) {
     // one-warp CTAs wait for the kernel before: started beside it they would
     // take the places it leaves, unevenly over the sub-partitions
     if (ntiles <= 4ull * sms) return {(int)(ntiles ? ntiles : 1), 32, sms, false};
-    return {sms * per_sm, 32 * kWideWarps, sms, true};
+    return {sms * per_sm, 32 * kWideWarps, sms, ntiles < kOverlapTiles};
 }
 
 }  // namespace tdes

@@ -76,6 +76,13 @@ __device__ __forceinline__ void wait_for_primary() {
 
 constexpr int kTileBlocks = 1024;  // blocks per warp tile: 32 lanes x 32 blocks
 constexpr int kWideWarps = 8;      // warps per CTA for large inputs
+// A call of so many tiles (512 MiB, 1.2 ms) neither starts beside the kernel before
+// nor lets the next start beside it: the next one's CTAs, waiting, take every place
+// that its own leave.  Beside a row of 1 GiB calls, a small call on another stream
+// waited for a whole kernel each time (2.4 ms, the first 3.3); so it waits until the
+// kernel's first CTAs end (after 1.3 ms), and from then on 0.05 to 0.1 ms.  The row
+// takes 3 to 9 us a call longer (ECB 2441 -> 2445).
+constexpr uint32_t kOverlapTiles = 1u << 16;
 constexpr int kTableWords = 3328;  // words of one bitsliced round-constant table
 constexpr int kChunkBytes = 384;   // 48 rounds x 8 six-bit round-key groups
 

@@ -225,7 +225,7 @@ tdes_ecb_kernel(const uint32_t* __restrict__ table, const uint8_t* in, uint8_t* 
     __shared__ __align__(16) uint32_t tab[table_words<STAGES>()];
     extern __shared__ __align__(16) uint4 ecb_data[];  // kCtrWarpBytes per warp (VEC only)
     __shared__ uint32_t slots[kWideWarps];
-    launch_dependents();
+    if (nblocks < (uint64_t)kOverlapTiles * kTileBlocks) launch_dependents();
     stage_table<STAGES>(tab, table);
     publish_slot(slots);
     __syncthreads();
@@ -361,7 +361,7 @@ tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr
     __shared__ __align__(16) uint32_t tab[table_words<STAGES>()];
     extern __shared__ __align__(16) uint4 ctr_data[];  // kCtrWarpBytes per warp
     __shared__ uint32_t slots[kWideWarps];
-    launch_dependents();
+    if (nblocks < (uint64_t)kOverlapTiles * kTileBlocks) launch_dependents();
     stage_table<STAGES>(tab, table);
     publish_slot(slots);
     __syncthreads();
@@ -496,7 +496,7 @@ tdes_cbc_dec_kernel(const uint32_t* __restrict__ table, uint64_t iv, const uint8
     __shared__ __align__(16) uint32_t tab[table_words<STAGES>()];
     extern __shared__ __align__(16) uint4 cbc_data[];  // kCtrWarpBytes per warp (VEC only)
     __shared__ uint32_t slots[kWideWarps];
-    launch_dependents();
+    if (nblocks < (uint64_t)kOverlapTiles * kTileBlocks) launch_dependents();
     stage_table<STAGES>(tab, table);
     publish_slot(slots);
     __syncthreads();
