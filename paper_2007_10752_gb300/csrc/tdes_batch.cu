@@ -61,8 +61,12 @@ constexpr uint64_t kMixedSplitBlocks = 128 * 1024;
 constexpr uint64_t kSoloChainBlocks = 512;                // longer CBC-enc chains: one per warp
 // What the choice for shorter chains weighs, in ns: a block of a chain that a
 // warp walks alone (one such chain per SM sub-partition at a time), a block of
-// one of 32 that share a warp, and a tile's share of a sub-partition.
-constexpr uint64_t kSoloBlockNs = 800, kPackedBlockNs = 4000, kTileNs = 12000;
+// one of 32 that share a warp, and a tile's share of a sub-partition.  A solo
+// chain's tables take as long as eight of its blocks.
+constexpr uint64_t kSoloBlockNs = 800, kPackedBlockNs = 4000, kTileNs = 12000, kSoloTableBlocks = 8;
+// A block of packed chains for each packed warp on the SM (their table lookups bind
+// them): CTAs of packed chains alone have 8, two CTAs on an SM 16.
+constexpr uint64_t kPackedWarpNs = 810;
 constexpr uint64_t kSubPartitions = 608;
 constexpr int kPerKeyWords = 2 * TDES_TABLE_WORDS;        // enc + dec bitsliced tables
 constexpr int kPerKeyChunks = 2 * TDES_SUBKEY_WORDS;      // enc + dec scalar groups
@@ -786,16 +790,37 @@ void build_plan(const tdes_desc_t* descs, uint32_t count, uint32_t key_count, in
     // keeps its packed chains, and with them the kernel without slots).  4096
     // records of 64 B to 4 KiB, 411 of them chains: 2.87 -> 1.21 ms a ticket,
     // with the wider grid and the overlapped mixed-key kernel of enqueue_batch.
-    uint64_t solo_blocks = 0;
-    for (uint32_t i = 0; i < h->n_c_solo; ++i) solo_blocks += msgs[c_list[i]].nblocks;
+    uint64_t solo_blocks = 0;  // with the tables of those past a sub-partition's first
+    auto take_solo = [&](uint32_t i) {
+        solo_blocks += msgs[c_list[i]].nblocks + (i >= kSubPartitions ? kSoloTableBlocks : 0);
+    };
+    for (uint32_t i = 0; i < h->n_c_solo; ++i) take_solo(i);
+    const uint32_t long_chains = h->n_c_solo;
     const uint64_t tiles_ns = b_prefix.back() * kTileNs / kSubPartitions;
+    auto solo_ns = [&] {
+        return h->n_c_solo ? std::max(msgs[c_list[0]].nblocks, solo_blocks / kSubPartitions) * kSoloBlockNs
+                           : 0;
+    };
+    const uint64_t long_ns = solo_ns();
     for (; h->n_c_solo < h->n_c; ++h->n_c_solo) {
         const uint64_t nb = msgs[c_list[h->n_c_solo]].nblocks;
-        const uint64_t solo_ns =
-            h->n_c_solo ? std::max(msgs[c_list[0]].nblocks, solo_blocks / kSubPartitions) * kSoloBlockNs
-                        : 0;
-        if (nb * kPackedBlockNs <= std::max<uint64_t>({tiles_ns, solo_ns, 10000})) break;
-        solo_blocks += nb;
+        if (nb * kPackedBlockNs <= std::max<uint64_t>({tiles_ns, solo_ns(), 10000})) break;
+        take_solo(h->n_c_solo);
+    }
+    // Beside many packed chains the solo ones' table reads wait behind their
+    // lookups (a block of a solo chain 0.8 -> 2 us with two packed warps on an SM):
+    // then all of them packed may end sooner.  20000 chains of 3, 10, 50 and 200
+    // blocks: 36, 79, 323 and 1246 us; without this 60, 118, 502 and 1980 us.  60000
+    // of 10 and 50, where some go alone: 129 and 585 us, all packed 151 and 657.
+    const uint64_t packed = (h->n_c - h->n_c_solo + 31) / 32, all = (h->n_c - long_chains + 31) / 32;
+    if (h->n_c_solo > long_chains && packed) {
+        const uint64_t sms = kSubPartitions / 4, most = 2 * sms;
+        const uint64_t slowed = (solo_ns() + kSoloTableBlocks * kSoloBlockNs) *
+                                (10 * most + 14 * std::min(packed, most)) / (10 * most);
+        const uint64_t rest = msgs[c_list[h->n_c_solo]].nblocks * kPackedWarpNs *
+                              std::max<uint64_t>(4, (packed + sms - 1) / sms);
+        const uint64_t none = msgs[c_list[long_chains]].nblocks * kPackedWarpNs * (all > 8 * sms ? 16 : 8);
+        if (std::max(slowed, rest) >= std::max(none, long_ns)) h->n_c_solo = long_chains;
     }
     h->n_c_items = h->n_c_solo + (h->n_c - h->n_c_solo + 31) / 32;
     h->n_b = (uint32_t)b_msg.size();

@@ -108,3 +108,19 @@ def test_small_calls_between_wide_ones(cuda_lib):
     wide, many, one = call(1100), call(2), call(1 / 16)
     r = _ratio(lambda: (many(), wide()), lambda: (one(), wide()), rows=20, rounds=20)
     assert r <= 1.15, r
+
+
+@pytest.mark.parametrize("nb,limit", [(3, 2.4), (50, 7.0), (200, 8.0)], ids=str)
+def test_many_short_chains(cuda_lib, nb, limit):
+    """20000 CBC encryptions of nb blocks against 32 of them: packed 32 to a warp
+    they take 1.8, 5.5 and 6.7 times as long, where most go alone 3, 8.6 and 10.6."""
+    n = 20000
+    src = torch.zeros(8 * nb * n, dtype=torch.uint8, device="cuda")
+    synth.fill_device(src, nb)
+    dst = torch.empty_like(src)
+    kt = cuda_lib.KeyTable(synth.key_triples(nb, 64))
+    many, few = (cuda_lib.Batch(kt, [(4, i % 64, i << 32, src.data_ptr() + 8 * nb * i,
+                                      dst.data_ptr() + 8 * nb * i, 8 * nb) for i in range(count)])
+                 for count in (n, 32))
+    r = _ratio(many.launch_graph, few.launch_graph, rounds=20)
+    assert r <= limit, r
