@@ -53,24 +53,22 @@ constexpr int kMixedWarpBytes = kUniTableBytes + 32 * kSliceSlots * 4 + 32;
 // read again after the rounds
 constexpr int kTileSlots = 128;
 constexpr int kTileWarpBytes = kUniTableBytes + kTileSlots * 4;
-// CBC-encryption chains: a warp's table, its 1024 chains' message indices and
-// one held block per chain (25 KB; one CTA per SM of 8 warps for mixed-key
-// chains, 9 for single-key tiles)
+// Single-key CBC-encryption tiles: a warp's table, its 1024 chains' message
+// indices and one held block per chain (25 KB; one CTA of 9 warps per SM)
 constexpr int kChainWarpBytes = kUniTableBytes + 32 * 32 * 4 + 32 * 32 * 8;
 // Mixed-key CBC-encryption slices: 6 warps per CTA, each warp with its table
 // and its chains' message indices in shared memory (17 KB) and its held blocks
-// in a slab of global scratch (8 KB per warp).  Two launches of a CTA per SM
-// make 12 warps of them, and a CTA fits beside a tile kernel's.
+// in a slab of global scratch (8 KB per warp).  One CTA per SM before the tiles
+// or two after them (chains_first).
 constexpr int kMixedChainWarps = 6;
 constexpr int kMixedChainWarpBytes = kUniTableBytes + 32 * 32 * 4;
-constexpr int kMaxChainCtas = 256;  // the kernel's grid: min(SMs, this)
+constexpr int kMaxChainCtas = 256;  // a CTA per SM: min(SMs, this)
 // sm_103a shared memory: 228 KB per SM, 1 KB of it reserved per resident CTA,
 // so a CTA may take at most 227 KB
 constexpr int kSmemPerSm = 228 * 1024, kSmemReservedPerCta = 1024;
 static_assert(kKeyChainWarps * kChainWarpBytes + kSmemReservedPerCta <= kSmemPerSm, "single-key chain CTA");
-static_assert(kMixedChainWarps * kMixedChainWarpBytes + kUniWarps * kMixedWarpBytes +
-                      2 * kSmemReservedPerCta <= kSmemPerSm,
-              "a mixed-key chain CTA beside a tile CTA");
+static_assert(2 * (kMixedChainWarps * kMixedChainWarpBytes + kSmemReservedPerCta) <= kSmemPerSm,
+              "two mixed-key chain CTAs per SM");
 static_assert(2 * (kUniWarps * kTileWarpBytes + kSmemReservedPerCta) <= kSmemPerSm, "two tile CTAs per SM");
 static_assert(2 * (kUniWarps * kMixedWarpBytes + kSmemReservedPerCta) <= kSmemPerSm,
               "two mixed-key CTAs per SM");
@@ -727,13 +725,28 @@ __global__ void __launch_bounds__(KIND == kKindCbcEnc ? 32 * kKeyChainWarps : 32
     first_cta_waits();
 }
 
+// Whether the chain tiles run before the other work kernels.  A chain tile takes a
+// warp long after the other tiles of its size are done, so few chain tiles, one for
+// each warp at most, start first and overlap with the rest on the SMs they leave:
+// 10% chains under 4096 keys, 64 MB of 64-byte messages 833 us last, 546 first; 512
+// MB 2333 and 2236; 1 GB of 256-byte ones 4457 and 3588.  More tiles than that
+// want all 12 warps of an SM, which they have last: a tile CTA finds no place beside
+// a chain CTA (two warps of each on a sub-partition take more than its registers), so
+// first they would run with 6 and hold up the tiles (under 65536 keys 64 MB 885 us
+// last, 1056 first, 1 GB of 256-byte messages 5833 and 6624; chains alone, 1 GB of
+// 128-byte messages, 5272 and 6640).
+__device__ __forceinline__ bool chains_first(uint32_t ntiles, uint32_t ctas) {
+    return ntiles <= ctas * kMixedChainWarps;
+}
+
 // Mixed-key tiles: slice s of tile t is slice first + 32 t + s; lane s works
 // out its slice's first message position, count and mode and loads its
 // key's packed table row, and a transpose across the lanes builds the tile's
 // table (bit s of every word: slice s's key and direction).  Slices differ
 // in mode, but each slice's mode is the same in every lane.
-// Chain tiles are claimed from a counter, by both launches of the kernel (late:
-// the second).
+// Chain tiles are claimed from a counter.  The chain kernel is launched twice, with
+// a CTA per SM before the other work kernels and with two after them (late), and
+// one of the launches does all the work (chains_first).
 template <bool CHAIN>
 __global__ void __launch_bounds__(CHAIN ? 32 * kMixedChainWarps : 32 * kUniWarps, 2)
     uni_mixed_kernel(UniParams p, uint32_t late) {
@@ -746,8 +759,10 @@ __global__ void __launch_bounds__(CHAIN ? 32 * kMixedChainWarps : 32 * kUniWarps
     const uint32_t ns = CHAIN ? p.hdr->slices[1] : p.hdr->slices[0];
     const uint32_t ntiles = (ns + 31u) / 32u;
     const uint32_t W = gridDim.x * kWarps;
+    const bool mine = !CHAIN || chains_first(ntiles, late ? gridDim.x / 2 : gridDim.x) == (late == 0);
     auto claim = [&](uint32_t t) {  // the tile after t
         if (!CHAIN) return t + W;
+        if (!mine) return ntiles;
         uint32_t c = 0;
         if (lane == 0) c = atomicAdd(&p.hdr->chain_next, 1u);
         return __shfl_sync(0xFFFFFFFFu, c, 0);
@@ -794,8 +809,8 @@ __global__ void __launch_bounds__(CHAIN ? 32 * kMixedChainWarps : 32 * kUniWarps
                 A1[s] = c.y;
             }
             uni_chain_passes<true>(p, A0, A1, wtab, widx,
-                                   p.held + (size_t)((2u * blockIdx.x + late) * kWarps + warp) * (32 * 32),
-                                   lane, false);
+                                   p.held + (size_t)(blockIdx.x * kWarps + warp) * (32 * 32), lane,
+                                   false);
         } else {
             // lane l holds block l % m of the slice's message l / m.  With at
             // most kSliceSlots messages a slice, each message's index (written
@@ -1078,13 +1093,8 @@ int tdes_uniform_crypt(const tdes_keytable_t* kt, const uint32_t* key_index, con
     }
     if (e == cudaSuccess) {
         what = "work kernels";
-        // CBC-encryption chains of mixed-key slices: two launches of a CTA per
-        // SM, the first before the tiles, with its CTAs beside theirs: alone the
-        // chains keep the logic pipe half busy.  In larger calls the tiles' traffic
-        // drives the chains' messages out of L2 between passes, and both launches
-        // come last (64 B: 256 MB 1187 us first, 1469 us last; 1 GB 4113 and 3910
-        // us; 128 B: 1 GB 3674 and 3810 us; 256 B: 1 GB 3429 and 4327 us; 16 B: 64
-        // MB 648 and 712 us, 128 MB 1215 and 1173 us).
+        // CBC-encryption chains of mixed-key slices: launched before the tiles and
+        // after them, one of which does them (chains_first).
         // Their held blocks in a slab of global scratch, with accesses that ask
         // L2 to keep its lines, beat 8 warps with everything in shared memory
         // (2^28 messages of 64 B: 65.10 -> 64.20 ms); with the message indices
@@ -1097,15 +1107,13 @@ int tdes_uniform_crypt(const tdes_keytable_t* kt, const uint32_t* key_index, con
         const size_t dyn_mixed = (size_t)kUniWarps * kMixedWarpBytes;
         const size_t dyn_chain = (size_t)kMixedChainWarps * kMixedChainWarpBytes;
         const size_t dyn_key_chain = (size_t)kKeyChainWarps * kChainWarpBytes;
-        const bool chains_first = span <= (msg_bytes >= 32 ? msg_bytes << 23 : 64ull << 20);
         bool first = true;
         auto work = [&](unsigned ctas, int warps, size_t smem, auto kernel, auto... args) {
             if (e == cudaSuccess)
                 e = launch_kernel(kernel, ctas, 32 * warps, smem, s, !first, args...);
             first = false;
         };
-        if (chains_first)
-            work(chain_ctas, kMixedChainWarps, dyn_chain, uni_mixed_kernel<true>, p, 0u);
+        work(chain_ctas, kMixedChainWarps, dyn_chain, uni_mixed_kernel<true>, p, 0u);
         work(work_grid, kUniWarps, dyn,
              vec16 ? uni_tile_kernel<kKindEcb, true> : uni_tile_kernel<kKindEcb, false>, p);
         work(work_grid, kUniWarps, dyn,
@@ -1113,9 +1121,7 @@ int tdes_uniform_crypt(const tdes_keytable_t* kt, const uint32_t* key_index, con
         work(work_grid, kUniWarps, dyn,
              vec16 ? uni_tile_kernel<kKindCbcDec, true> : uni_tile_kernel<kKindCbcDec, false>, p);
         work(work_grid, kUniWarps, dyn_mixed, uni_mixed_kernel<false>, p, 0u);
-        if (!chains_first)
-            work(chain_ctas, kMixedChainWarps, dyn_chain, uni_mixed_kernel<true>, p, 0u);
-        work(chain_ctas, kMixedChainWarps, dyn_chain, uni_mixed_kernel<true>, p, 1u);
+        work(2 * chain_ctas, kMixedChainWarps, dyn_chain, uni_mixed_kernel<true>, p, 1u);
         work(geo.sms, kKeyChainWarps, dyn_key_chain, uni_tile_kernel<kKindCbcEnc, false>, p);
     }
     if (e == cudaSuccess && skipped != nullptr) {

@@ -136,3 +136,28 @@ def test_single_des_chain(cuda_lib):
     r = _ratio(lambda: cuda_lib.tdes_cbc_encrypt(des, 3, x, y),
                lambda: cuda_lib.tdes_cbc_encrypt(ede, 3, x, y), rounds=20)
     assert r <= 0.425, r
+
+
+# shares of the modes in tenths; the calls under many keys against under fewer: 1.08 and
+# 1.21 times as long, where chains that want all warps run first 1.28 and 1.49
+@pytest.mark.parametrize("msg,modes,many,few,limit", [
+    (64, [4] * 10, 65536, 4096, 1.18), (256, [0, 0, 0, 0, 2, 2, 2, 3, 3, 4], 65536, 16384, 1.35)],
+    ids=["chains", "mix"])
+def test_uniform_chains_under_many_keys(cuda_lib, msg, modes, many, few, limit):
+    n, T = 1 << 20, cuda_lib
+    words = lambda stream: torch.from_numpy(synth.u64s(msg, n, stream).view(np.int64)).cuda()  # noqa: E731
+    mode = torch.tensor(modes, dtype=torch.uint8, device="cuda")[(words(synth.STREAM_MODE) & 0xFFFF) * 10 >> 16]
+    iv = words(synth.STREAM_IV) & -(1 << 32)
+    src = torch.empty(n * msg, dtype=torch.uint8, device="cuda")
+    synth.fill_device(src, msg)
+    dst, pick, calls = torch.empty_like(src), words(synth.STREAM_KEYPICK), []
+    for keys in (many, few):
+        kt = T.KeyTable(synth.key_triples(msg, keys))
+        index = (pick & (keys - 1)).to(torch.int32)
+        need = T.tdes_uniform_scratch_bytes(kt, n, msg)
+        buf = torch.empty(need + 256, dtype=torch.uint8, device="cuda")
+        scratch = buf[-buf.data_ptr() % 256:][:need]
+        calls.append(lambda kt=kt, index=index, scratch=scratch: T.tdes_uniform_crypt(
+            kt, index, mode, iv, src, dst, msg, scratch=scratch))
+    r = _ratio(*calls, rounds=16)
+    assert r <= limit, r
