@@ -355,8 +355,9 @@ int tdes_cbc_encrypt(const tdes_ks_t* ks, uint64_t iv, const void* in, void* out
 // is a sixteenth of the call, but at least 8 MiB or a quarter of it: the first
 // copy in, the last kernel and the last copy out overlap with nothing, and
 // chunks below 8 MiB lose more in the gaps between copies.  With 32 MiB chunks
-// for every call: 16 MiB 284 us, 64 MiB 685 us, 256 MiB 1927 us; now 216, 575
-// and 1892 us (1 GiB takes 32 MiB chunks as before).
+// for every call, and so, medians of 15 in four processes by turns: 16 MiB 284 and 217
+// us, 64 MiB 692 and 572, 128 MiB 1105 and 1035, 256 MiB 1931 and 1893, the last a
+// gain that a busier host hides (1 GiB takes 32 MiB chunks either way).
 constexpr int kHostBufs = 16;
 
 int tdes_ecb_crypt_host(const tdes_ks_t* ks, int decrypt, const void* host_in, void* host_out,

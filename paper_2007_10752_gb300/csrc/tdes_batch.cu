@@ -58,7 +58,7 @@ constexpr uint64_t kSplitBlocks = 512;
 // 4096 records of 64 B to 4 KiB through a context 909 -> 861 us, the 4096-message
 // batch 3482 -> 3461 us, the server's closed loop 391 -> 402 GB/s.
 constexpr uint64_t kMixedSplitBlocks = 128 * 1024;
-constexpr uint64_t kSoloChainBlocks = 512;                // longer CBC-enc chains: one per warp
+constexpr uint64_t kSoloChainBlocks = 512;                // longer CBC-enc chains: always one per warp
 // What the choice for shorter chains weighs, in ns: a block of a chain that a
 // warp walks alone (one such chain per SM sub-partition at a time), a block of
 // one of 32 that share a warp, and a tile's share of a sub-partition.  A solo
@@ -67,7 +67,7 @@ constexpr uint64_t kSoloBlockNs = 800, kPackedBlockNs = 4000, kTileNs = 12000, k
 // A block of packed chains for each packed warp on the SM (their table lookups bind
 // them): CTAs of packed chains alone have 8, two CTAs on an SM 16.
 constexpr uint64_t kPackedWarpNs = 810;
-constexpr uint64_t kSubPartitions = 608;
+constexpr uint64_t kSubPartitions = 608;  // the GB300's: a plan is built without a device
 constexpr int kPerKeyWords = 2 * TDES_TABLE_WORDS;        // enc + dec bitsliced tables
 constexpr int kPerKeyChunks = 2 * TDES_SUBKEY_WORDS;      // enc + dec scalar groups
 constexpr int kWarpSmemBytes = TDES_TABLE_WORDS * 4;      // one table per warp (13 KB)
@@ -351,9 +351,9 @@ __device__ __forceinline__ bool mixed_slot(const BatchParams& p, const MSlice& s
     return true;
 }
 
-// One mixed-key tile of small messages (ECB, CTR, CBC decryption).  Slice s
-// (bit position s of every plane) carries up to 32 blocks under its own key
-// and direction, one per lane; its table bits come from the key table's
+// One mixed-key tile (ECB, CTR, CBC decryption).  Slice s (bit position s of every
+// plane) carries up to 32 blocks, of small messages or a piece of a medium one, under
+// its own key and direction, one per lane; its table bits come from the key table's
 // packed copy, lane s loading slice s's row, and a transpose across the lanes
 // turns 32 rows into 32 table words.
 __device__ __forceinline__ void batch_mixed_tile(const BatchParams& p, uint32_t tile,
@@ -435,8 +435,8 @@ __device__ __forceinline__ void batch_mixed_tile(const BatchParams& p, uint32_t 
 
 // The mixed-key tiles of a plan, in a kernel of their own launched just
 // before the persistent kernel: inside it, their code slowed the persistent
-// kernel's other paths by 4% (alternating A/B runs on the 4096-message batch,
-// which has no mixed-key tiles).  Warps stride over the tiles.
+// kernel's other paths by 4% (alternating A/B runs on the 4096-message batch
+// while it had no mixed-key tiles).  Warps stride over the tiles.
 __device__ __forceinline__ unsigned long long global_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -542,7 +542,7 @@ __device__ __noinline__ void batch_cbc_enc_item(const BatchParams& p, uint32_t i
     __syncwarp();
 }
 
-// SOLO_SLOTS: the plan has chains over 512 blocks, each walked by one warp.
+// SOLO_SLOTS: the plan has chains that are each walked by one warp.
 // They are latency-bound, and two on one SM sub-partition (SMSP) slow each
 // other down (a 4096-message batch: 865 against 517 ms), so each is taken
 // only by a warp that holds its SMSP's slot (%smid, %warpid: a placement hint
@@ -944,7 +944,7 @@ cudaError_t enqueue_batch(const BatchParams& p_in, uint64_t total_items, bool ne
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     p.times_end_in_mixed = total_items == 0;
-    if (p.n_m_tiles) {  // small messages of their own keys: disjoint from the rest
+    if (p.n_m_tiles) {  // other messages than the rest's
         // few tiles: one warp per CTA spreads them over the SM sub-partitions
         // (40 tiles alone: 97 -> 65 us)
         const int mw = p.n_m_tiles <= kSubPartitions ? 1 : warps;

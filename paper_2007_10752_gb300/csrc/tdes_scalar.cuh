@@ -77,9 +77,9 @@ TDES_HD uint64_t permute64_nib(uint64_t v, const uint64_t* __restrict__ tab) {
 }
 
 // The same EDE3 block as tdes_block_scalar with the permutations by nibble
-// tables (ipn/fpn: 16 x 16 words each) instead of bit loops; the host check's
-// form (the kernels take tdes_block_scalar_swap).  The 16 rounds
-// of a DES pass are unrolled by two so that the halves alternate in place,
+// tables (ipn/fpn: 16 x 16 words each) instead of bit loops: a form of the host
+// check alone, which no kernel takes (they take tdes_block_scalar_swap).  The 16
+// rounds of a DES pass are unrolled by two so that the halves alternate in place,
 // and each round's key words are loaded one round ahead, off the chain of
 // dependent operations that sets the latency of a block.
 template <int ROUNDS = 48>
@@ -110,7 +110,8 @@ TDES_HD uint64_t tdes_block_scalar_nib(uint64_t v, const uint32_t* __restrict__ 
 
 // IP and FP as swaps of bit groups between the halves: IP is a transpose of
 // the block's 8x8 bit matrix followed by a row reordering, and each of its
-// five steps exchanges one index bit.
+// five steps exchanges one index bit (the masked exchanges of Warren, "Hacker's
+// Delight", Sec. 7-3).
 TDES_HD void bit_swap(uint32_t& a, uint32_t& b, int n, uint32_t m) {
     const uint32_t t = ((a >> n) ^ b) & m;
     b ^= t;

@@ -79,7 +79,7 @@ struct Pending {
     uint64_t cost;
     bool stage;  // host buffers, large enough to be staged through the device
     bool alone;  // a long serial chain: batched on its own (see lone_request)
-    bool host;   // its input or its output is in host memory (of a group: of each request)
+    bool host;   // its input or its output is in host memory (in a group: so for every request)
 };
 
 // A batch takes requests until the input and output of those in device memory
@@ -91,11 +91,13 @@ struct Pending {
 // nothing (closed loop 131.5 GB/s so, 129.7 where they count).
 constexpr uint64_t kBatchCost = 32ull << 20;
 
-// Warps per SM for a batch whose requests all lie in host memory (none staged, no
-// serial chains, which want every warp): the host link is full with one warp on
-// each sub-partition, and more only queue on it, with the batches behind them.
-// Serving mix in pinned host memory, 12 -> 4 warps: p50 at 64 GB/s offered 0.068 ->
-// 0.056 ms, p99 0.61 -> 0.54, closed loop 132 -> 134 GB/s; with 8 warps p50 0.065.
+// Warps per SM (in whole CTAs) for a batch whose requests all read or write host
+// memory (none staged, no serial chains, which want every warp): the host link is
+// full with one warp on each sub-partition, and more only queue on it, with the
+// batches behind them.  Serving mix in pinned host memory, 12 -> 4 warps: p50 at 64
+// GB/s offered 0.068 -> 0.056 ms, p99 0.61 -> 0.54, closed loop 132 -> 134 GB/s; with 8
+// warps p50 0.065.  One side in host memory, p50 at 110 GB/s offered: to the device
+// 0.140 -> 0.117 ms, from it 0.092 -> 0.075, closed loops (151, 189 GB/s) as with 12.
 constexpr int kLinkWarps = 4;
 
 // A CBC-encryption request of more than 512 blocks is one serial chain that
@@ -316,7 +318,7 @@ struct tdes_server {
                 copy_in.clear();
                 copy_out.clear();
                 size_t staged = 0;
-                bool in_host = true;  // every request reads and writes host memory
+                bool in_host = true;  // every request reads or writes host memory, unstaged
                 for (size_t i = 0; i < take.size(); ++i) {
                     descs[i] = take[i].d;
                     in_host &= take[i].host && !take[i].stage;

@@ -25,8 +25,8 @@ swapped for the one its next use needs inside the same 3-input XOR that adds
 the S-box output, so the round key costs no extra logic operation.
 
 The kernels are bound by the logic pipe, so the round's time is its LOP3 count:
-169 S-box gates and 32 updates (1 GiB ECB: 2462 us with 170 gates, 2528 us with
-175, 2578 us with 181, same GPU).
+169 S-box gates and 32 updates (1 GiB ECB: 2460 us with 169 gates and 2532 us with
+175 in one run, 2527 us with 175 and 2578 us with 181 in another).
 
 Run:  python -m paper_2007_10752_gb300.gen.emit_cuda   (or emit() from build)
 """
