@@ -214,6 +214,10 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
 }
+__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(s), "l"(gmem) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
@@ -353,7 +357,10 @@ cudaError_t launch_ecb(const uint32_t* tab, const uint8_t* chunks, int stages, c
 // registers, directly as bit-planes (counter_planes: 3% fewer logic operations
 // a tile; 40 MB 118.8 -> 117.0 us).  The data tile the keystream is XORed into is copied into the
 // warp's 8 KiB of shared memory with cp.async before the rounds start, so
-// its memory latency hides behind them.
+// its memory latency hides behind them.  8-byte-aligned buffers take 8-byte
+// copies: loaded after the rounds, each load waits for the store before it (in
+// and out may be one buffer), 32 latencies in a row.  1 GiB there 2967 -> 2403 us
+// (single DES 1465 -> 914), 40 MB 129.7 -> 111.2.
 template <bool VEC, int STAGES>
 __global__ void __launch_bounds__(256, 2)
 tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr0,
@@ -372,7 +379,7 @@ tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr
     uint4* wbuf = ctr_data + (threadIdx.x >> 5) * (kCtrWarpBytes / 16);
     // Tile loop index and ragged-tile indexing: 64-bit for the 16-byte path
     // (measured 410 GB/s at 1 GiB against 399 with 32-bit indices there),
-    // 32-bit for the 8-byte-aligned variant (the 64-bit form spills there).
+    // 32-bit for the 8-byte-aligned variant (single DES, 96 MB: 90.6 us against 94.2).
     // Tile indices fit 32 bits: the host caps a call below 2^31 tiles.
     using Idx = typename std::conditional<VEC, uint64_t, uint32_t>::type;
     const Idx ntiles = (Idx)((nblocks + kTileBlocks - 1) / kTileBlocks);
@@ -384,23 +391,20 @@ tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr
 #pragma unroll
             for (int j = 0; j < 16; ++j) cp_async16(wbuf + 32 * j + lane, p + 32 * j);
             cp_async_commit();
-        }
-        uint32_t A0[32], A1[32];
-        if constexpr (VEC || STAGES == 1) {
-            counter_planes(nonce, ctr0 + (uint32_t)b0, lane, A0, A1);
-        } else {  // the 8-byte-aligned EDE3 variant would spill: words, transposed
-            const uint32_t nw = bswap32(nonce);
+        } else if (!VEC) {  // 32-bit in-tile indices
+            const uint2* p = reinterpret_cast<const uint2*>(in) + b0;
+            const uint32_t nvalid = (uint32_t)min((uint64_t)kTileBlocks, nblocks - b0);
 #pragma unroll
             for (int j = 0; j < 16; ++j)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const uint32_t b = (uint32_t)b0 + 2u * (32u * j + lane) + h;
-                    A0[2 * j + h] = nw;
-                    A1[2 * j + h] = bswap32(ctr0 + b);
+                    const uint32_t i = 2u * (32u * j + lane) + h;
+                    if (i < nvalid) cp_async8(reinterpret_cast<uint2*>(wbuf) + i, p + i);
                 }
-            transpose32(A0);
-            transpose32(A1);
+            cp_async_commit();
         }
+        uint32_t A0[32], A1[32];
+        counter_planes(nonce, ctr0 + (uint32_t)b0, lane, A0, A1);
         tdes_process32_planes<STAGES>(A0, A1, tab);
         if (full) {
             cp_async_wait_all();
@@ -424,8 +428,8 @@ tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr
                         __stcs(q + b, make_uint2(v.x ^ A0[2 * j + h], v.y ^ A1[2 * j + h]));
                     }
                 }
-        } else {  // 8-byte-aligned buffer: 32-bit in-tile indices
-            const uint2* p = reinterpret_cast<const uint2*>(in) + b0;
+        } else {
+            cp_async_wait_all();
             uint2* q = reinterpret_cast<uint2*>(out) + b0;
             const uint32_t nvalid = (uint32_t)min((uint64_t)kTileBlocks, nblocks - b0);
 #pragma unroll
@@ -434,7 +438,7 @@ tdes_ctr_kernel(const uint32_t* __restrict__ table, uint32_t nonce, uint32_t ctr
                 for (int h = 0; h < 2; ++h) {
                     const uint32_t i = 2u * (32u * j + lane) + h;
                     if (i < nvalid) {
-                        const uint2 v = __ldcs(p + i);
+                        const uint2 v = reinterpret_cast<const uint2*>(wbuf)[i];
                         __stcs(q + i, make_uint2(v.x ^ A0[2 * j + h], v.y ^ A1[2 * j + h]));
                     }
                 }
